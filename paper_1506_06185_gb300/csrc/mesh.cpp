@@ -78,19 +78,32 @@ const double* corner_pos(const HostMesh& m, const int c[3]) {
   return &m.vpos[(((size_t)c[2] * (m.sub[1] + 1) + c[1]) * (m.sub[0] + 1) + c[0]) * 3];
 }
 
-// Physical position of a local lattice node of a macro at refinement N: the
-// macro's corners P0..P3 (moved corners), P0 + (i (P1-P0) + j (P2-P0) +
-// k (P3-P0)) / N; else the unit-cube grid position mapped by G.
-void position(const HostMesh& m, int macro, int N, int i, int j, int k, double out[3]) {
+// Physical vector between two local lattice nodes of a macro at refinement N
+// whose lattice coordinates differ by (i, j, k): (i (P1 - P0) + j (P2 - P0) +
+// k (P3 - P0)) / N with the macro's corners P0..P3 (moved corners), else the
+// difference of the unit-cube grid positions mapped by G.  The element
+// matrices are built from these vectors and not from differences of rounded
+// positions: the latter are off by eps * N * sub of an edge, which on cubes
+// with an odd number of sub-cubes (spacing 1/3) left weights of 1e-13 on the
+// eight directions that vanish, and such meshes ran the 15-point kernels.
+// (The host code is compiled without contraction to fused multiply-adds: a b
+// - c d of equal products has to be 0 on every machine.)
+void offset_vector(const HostMesh& m, int macro, int N, int i, int j, int k, double out[3]) {
+  const double *P0, *P1, *P2, *P3;
   if (!m.mverts.empty()) {
-    const double* P[4];
-    for (int q = 0; q < 4; ++q) P[q] = &m.vpos[3 * (size_t)m.mverts[macro][q]];
-    for (int a = 0; a < 3; ++a)
-      out[a] = P[0][a] + (i * (P[1][a] - P[0][a]) + j * (P[2][a] - P[0][a]) + k * (P[3][a] - P[0][a])) / N;
-    return;
-  }
-  if (!m.vpos.empty()) {
+    P0 = &m.vpos[3 * (size_t)m.mverts[macro][0]];
+    P1 = &m.vpos[3 * (size_t)m.mverts[macro][1]];
+    P2 = &m.vpos[3 * (size_t)m.mverts[macro][2]];
+    P3 = &m.vpos[3 * (size_t)m.mverts[macro][3]];
+  } else {
     const MacroGeo& g = m.geo[macro];
+    if (m.vpos.empty()) {
+      double p[3];
+      for (int a = 0; a < 3; ++a)
+        p[a] = double(i * g.e1[a] + j * g.e2[a] + k * g.e3[a]) / (double(m.sub[a]) * N);
+      for (int a = 0; a < 3; ++a) out[a] = m.G[3 * a] * p[0] + m.G[3 * a + 1] * p[1] + m.G[3 * a + 2] * p[2];
+      return;
+    }
     int c[4][3];
     for (int a = 0; a < 3; ++a) {
       c[0][a] = g.v0[a];
@@ -98,22 +111,16 @@ void position(const HostMesh& m, int macro, int N, int i, int j, int k, double o
       c[2][a] = g.v0[a] + g.e2[a];
       c[3][a] = g.v0[a] + g.e3[a];
     }
-    const double* P0 = corner_pos(m, c[0]);
-    const double* P1 = corner_pos(m, c[1]);
-    const double* P2 = corner_pos(m, c[2]);
-    const double* P3 = corner_pos(m, c[3]);
-    for (int a = 0; a < 3; ++a)
-      out[a] = P0[a] + (i * (P1[a] - P0[a]) + j * (P2[a] - P0[a]) + k * (P3[a] - P0[a])) / N;
-    return;
+    P0 = corner_pos(m, c[0]);
+    P1 = corner_pos(m, c[1]);
+    P2 = corner_pos(m, c[2]);
+    P3 = corner_pos(m, c[3]);
   }
-  int64_t X[3];
-  local_to_fine(m.geo[macro], N, i, j, k, X);
-  double p[3] = {double(X[0]) / (double(m.sub[0]) * N), double(X[1]) / (double(m.sub[1]) * N),
-                 double(X[2]) / (double(m.sub[2]) * N)};
-  for (int a = 0; a < 3; ++a) out[a] = m.G[3 * a] * p[0] + m.G[3 * a + 1] * p[1] + m.G[3 * a + 2] * p[2];
+  for (int a = 0; a < 3; ++a)
+    out[a] = (i * (P1[a] - P0[a]) + j * (P2[a] - P0[a]) + k * (P3[a] - P0[a])) / N;
 }
 
-// P1 stiffness of one tetrahedron with unit coefficient: gradients of the
+// P1 stiffness of one tetrahedron (vertices relative to any origin) with unit coefficient: gradients of the
 // barycentric coordinates from the inverse edge matrix, times the volume.
 void tet_stiffness(const double X[4][3], double K[4][4]) {
   double E[3][3];
@@ -200,7 +207,7 @@ void class_weights(const HostMesh& m, int macro, int N, int mask, double w[NDIR]
         L[q][0] = a - b;
         L[q][1] = b - c;
         L[q][2] = c;
-        position(m, macro, N, L[q][0], L[q][1], L[q][2], X[q]);
+        offset_vector(m, macro, N, L[q][0] - i, L[q][1] - j, L[q][2] - k, X[q]);
       }
       if (!inside) continue;
       double K[4][4];
