@@ -345,10 +345,11 @@ int hhg_batch_info(hhg_batch* batch, int64_t* info);
  * running: for example a host application that hands the device's memory to
  * its own arena allocator at start-up, or code on a path where device
  * allocation is forbidden.  This call runs the same global V(pre, post) cycle
- * as hhg_vcycle (without the residual norm) but its coarse-grid CG keeps its
- * work vectors in a fixed array of the library's static device memory
+ * as hhg_vcycle (without the residual norm) but its coarse-grid CG takes the
+ * work vectors that do not fit its shared memory from a fixed array of the
+ * library's static device memory
  * (4 x 16384 doubles = 512 KiB, which every GPU that loads the library holds
- * until the process exits) instead of in memory obtained from cudaMalloc; the
+ * until the process exits) instead of from memory obtained from cudaMalloc; the
  * call itself makes no cudaMalloc, cudaFree or other allocating call.
  * Limit: the coarsest level may have at most 16384 unknowns; larger meshes
  * get HHG_ERR_ARG.  Meshes of general connectivity are accepted.  The mesh's

@@ -406,6 +406,8 @@ int upload_problem(hhg_mesh* m, const HostProblem& h, DevProblem& d) {
   }
   d.n_cg = h.n_cg;
   d.nnz = (int64_t)h.val.size();
+  d.cg_width = 0;
+  for (int q = 0; q < h.n_cg; ++q) d.cg_width = std::max(d.cg_width, h.rowptr[q + 1] - h.rowptr[q]);
   HHG_TRY(upload(m, &d.rowptr, h.rowptr));
   HHG_TRY(upload(m, &d.col, h.col));
   HHG_TRY(upload(m, &d.val, h.val));

@@ -407,6 +407,7 @@ struct DevProblem {
   int64_t* udst = nullptr;
   int* umaster = nullptr;
   double* cg_work = nullptr;        // 4 * n_cg scratch
+  int cg_width = 0;                 // entries of the longest row
   double* partial = nullptr;        // per-CTA partial sums of the norm
   int n_partial = 0;
   double* scalar = nullptr;         // [4]: norm^2 result, cg info

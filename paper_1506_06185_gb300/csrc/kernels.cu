@@ -1803,27 +1803,176 @@ __device__ __forceinline__ double cta_sum(double v, double* sh) {
 }
 
 constexpr int CG_THREADS = 256;
+constexpr int CG_WARPS = CG_THREADS / 32;
 
-// Sum of v over the CTA (CG_THREADS threads), returned to every thread in the
-// same order (warp partials 0..7); buf holds the warp partials.  Consecutive
-// reductions alternate between two buffers.
-__device__ __forceinline__ double cg_allreduce(double v, double* buf) {
-  const int t = threadIdx.y * blockDim.x + threadIdx.x;   // 1-D or (32, 8) CTAs
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  if ((t & 31) == 0) buf[t >> 5] = v;
-  __syncthreads();
-  double s = 0.0;
+// Sum over the warp, the same bits in every lane: both partners of a step add
+// the same two rounded values (__dadd_rn keeps the compiler from fusing a
+// lane's own product into its first add).
+__device__ __forceinline__ double warp_sum_xor(double v) {
 #pragma unroll
-  for (int w = 0; w < CG_THREADS / 32; ++w) s += buf[w];
-  return s;
+  for (int o = 16; o > 0; o >>= 1) v = __dadd_rn(v, __shfl_xor_sync(0xffffffffu, v, o));
+  return v;
+}
+
+// The CG's sums have one order whatever the launch: rows in blocks of 32 (or
+// 128, see cg_block_shift), a block summed by the shuffle tree above (missing
+// rows count 0), block b added
+// to bucket b mod 32 in ascending order, the 32 buckets summed by the same
+// tree.  So the one-CTA form below (also run by the persistent batch executor
+// and the allocation-free cycle) and the cluster form give the same iterates
+// bit for bit.
+//
+// One CTA of CG_THREADS threads: warp w takes the blocks w, w + 8, ... and
+// holds the buckets w, w + 8, w + 16, w + 24 in acc.  buf: 32 doubles;
+// consecutive sums alternate between two buffers.
+__device__ __forceinline__ double cg_allreduce(const double (&acc)[4], double* buf) {
+  const int t = threadIdx.y * blockDim.x + threadIdx.x;   // 1-D or (32, 8) CTAs
+  const int lane = t & 31, w = t >> 5;
+  if (lane < 4) buf[w + CG_WARPS * lane] = lane == 0 ? acc[0] : lane == 1 ? acc[1] : lane == 2 ? acc[2] : acc[3];
+  __syncthreads();
+  return warp_sum_xor(buf[lane]);
+}
+
+// Rows per lane of a block (as a shift): from 16385 rows on a block has 128
+// rows, lane l's rows l, l + 32, l + 64, l + 96 being added first, which
+// leaves a quarter of the tree's operations.
+__host__ __device__ __forceinline__ int cg_block_shift(int n) { return n > 16384 ? 2 : 0; }
+
+// Calls body(q) -> double for the rows q of the warp's blocks and returns the
+// sum over all rows (to every thread).
+template <class F>
+__device__ __forceinline__ double cg_rows_sum(int n, double* buf, F&& body) {
+  const int t = threadIdx.y * blockDim.x + threadIdx.x;
+  const int lane = t & 31, w = t >> 5;
+  const int sh = cg_block_shift(n);
+  const int nb = ((n - 1) >> (5 + sh)) + 1;
+  double acc[4] = {0.0, 0.0, 0.0, 0.0};
+  for (int b0 = w; b0 < nb; b0 += 32) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const int b = b0 + CG_WARPS * e;
+      if (b < nb) {
+        double v = 0.0;
+        for (int g = 0; g < 1 << sh; ++g) {
+          const int q = ((b << sh) + g) * 32 + lane;
+          if (q < n) v = g ? __dadd_rn(v, body(q)) : body(q);
+        }
+        acc[e] += warp_sum_xor(v);
+      }
+    }
+  }
+  return cg_allreduce(acc, buf);
+}
+
+// 1 / b, about one unit in the last place: the hardware's reciprocal
+// approximation y and one third-order step y (1 + e + e^2), e = 1 - b y
+// (Halley's iteration for 1 / b).  Three dependent FP64 operations of 68
+// clocks each where the IEEE division takes 590 clocks of latency; x and r
+// move by the same step, so its rounding only turns the search direction.
+// Operands near the ends of the exponent range take the IEEE division.
+__device__ __noinline__ double cg_recip_ieee(double b) { return 1.0 / b; }
+__device__ __forceinline__ double cg_recip(double b) {
+  const uint32_t e = ((uint32_t)__double2hiint(b) >> 20) & 0x7ffu;
+  if (e - 64u > 0x7ffu - 128u) return cg_recip_ieee(b);
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(b));
+  double d = fma(-b, y, 1.0);
+  d = fma(d, d, d);
+  return fma(y, d, y);
+}
+
+// The test sqrt(rr) > thr, set up once for a thr: rr (>= 0, or not a number) is
+// compared as an integer with thr^2 (1 +- 1e-14), and only between the two, or
+// where thr^2 is near the ends of the exponent range, the square root (650
+// clocks) is taken.
+struct CgTest {
+  double thr;
+  long long lo, hi;
+};
+__device__ __forceinline__ CgTest cg_test(double thr) {
+  CgTest t{thr, 0, 0x7ff0000000000000ll};
+  const double t2 = thr * thr;
+  if (t2 > 1e-280 && t2 < 1e280) {
+    t.lo = __double_as_longlong(t2 * (1.0 - 1e-14));
+    t.hi = __double_as_longlong(t2 * (1.0 + 1e-14));
+  }
+  return t;
+}
+__device__ __noinline__ bool cg_above_sqrt(double rr, double thr) { return sqrt(rr) > thr; }
+__device__ __forceinline__ bool cg_above(double rr, const CgTest& t) {
+  const long long b = __double_as_longlong(rr);
+  if (b > t.hi && b < 0x7ff0000000000000ll) return true;
+  if (b < t.lo) return false;
+  return cg_above_sqrt(rr, t.thr);
 }
 
 // CG on the compact free nodes of the coarsest level from x = 0 until
-// ||r|| <= rtol ||b|| or maxit iterations.  x, r, p and A p live in shared
-// memory (smem != 0) or in the global work array (4 n doubles).  Each
-// iteration: A p and p.Ap (one reduction), the updates of x and r and r.r
-// (one reduction), the new direction; row q belongs to thread q mod
-// CG_THREADS throughout.
+// ||r|| <= rtol ||b|| or maxit iterations.  The direction's image s = A p is
+// carried along, s <- A r + beta s, so that the product A r does not wait for
+// beta.  One iteration: p.s, alpha = r.r / p.s, x += alpha p, r -= alpha s,
+// r.r, beta = r.r / old r.r (times the reciprocal, formed beside the critical
+// path), p <- r + beta p, s <- A r + beta s.  A row's product is summed in two
+// chains, even and odd entries.
+//
+// One CTA of CG_THREADS threads; x, r, p and s live in shared or in global
+// memory (4 n doubles); a row belongs to one thread throughout.  red: 64
+// doubles of shared memory.
+template <class T>
+__device__ __forceinline__ void cg_one_cta(int n, const int* rowptr, const int* col, const double* val,
+                                           const int64_t* fsrc, const T* f, const T* fI, const int* uptr,
+                                           const int64_t* udst, const int* umaster, T* u, T* uI, double* x, double* r,
+                                           double* p, double* s, double rtol, int maxit, int* iters, double* red) {
+  const int t = threadIdx.y * blockDim.x + threadIdx.x;
+  auto row_times = [&](int q) {
+    double a0 = 0.0, a1 = 0.0;
+    const int e1 = rowptr[q + 1];
+    for (int e = rowptr[q]; e < e1; e += 2) {
+      a0 = fma(val[e], r[col[e]], a0);
+      if (e + 1 < e1) a1 = fma(val[e + 1], r[col[e + 1]], a1);
+    }
+    return a0 + a1;
+  };
+  double rr = cg_rows_sum(n, red, [&](int q) {
+    const int64_t src = fsrc[q];
+    const double b = src >= 0 ? (double)f[src] : (double)fI[-1 - src];
+    x[q] = 0.0;
+    r[q] = b;
+    return b * b;
+  });
+  const double bnorm = sqrt(rr);
+  const CgTest test = cg_test(rtol * bnorm);
+  int it = 0;
+  double beta = 0.0;
+  while (bnorm > 0.0 && it < maxit && cg_above(rr, test)) {
+    // every r entry was written before the barrier of the last sum
+    const double pAp = cg_rows_sum(n, red + 32, [&](int q) {
+      const double w = row_times(q);
+      const double pq = it ? fma(beta, p[q], r[q]) : r[q];
+      const double sq = it ? fma(beta, s[q], w) : w;
+      p[q] = pq;
+      s[q] = sq;
+      return pq * sq;
+    });
+    const double alpha = rr * cg_recip(pAp);
+    const double inv = cg_recip(rr);
+    const double rr_new = cg_rows_sum(n, red, [&](int q) {
+      x[q] = fma(alpha, p[q], x[q]);
+      const double rq = fma(-alpha, s[q], r[q]);
+      r[q] = rq;
+      return rq * rq;
+    });
+    beta = rr_new * inv;
+    rr = rr_new;
+    ++it;
+  }
+  for (int q = t; q < n; q += CG_THREADS) {
+    const T v = (T)x[q];
+    for (int e = uptr[q]; e < uptr[q + 1]; ++e) u[udst[e]] = v;
+    if (umaster[q] >= 0) uI[umaster[q]] = v;
+  }
+  if (t == 0 && iters) *iters = it;
+}
+
 template <class T>
 __global__ void __launch_bounds__(CG_THREADS) k_cg(int n, const int* __restrict__ rowptr, const int* __restrict__ col,
                                                    const double* __restrict__ val, const int64_t* __restrict__ fsrc,
@@ -1831,58 +1980,288 @@ __global__ void __launch_bounds__(CG_THREADS) k_cg(int n, const int* __restrict_
                                                    const int* __restrict__ uptr, const int64_t* __restrict__ udst,
                                                    const int* __restrict__ umaster, T* __restrict__ u,
                                                    T* __restrict__ uI, double* __restrict__ work, double rtol,
-                                                   int maxit, int* __restrict__ iters, int smem) {
+                                                   int maxit, int* __restrict__ iters) {
+  __shared__ double red[64];
+  cg_one_cta<T>(n, rowptr, col, val, fsrc, f, fI, uptr, udst, umaster, u, uI, work, work + n, work + 2 * (size_t)n,
+                work + 3 * (size_t)n, rtol, maxit, iters, red);
+}
+
+// --- the same CG on a thread-block cluster --------------------------------
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ uint32_t cluster_map(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ double cluster_load(uint32_t addr) {
+  double v;
+  asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(addr));   // ordered by the barriers' asm
+  return v;
+}
+__device__ __forceinline__ void cluster_store(uint32_t addr, double v) {
+  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(addr), "d"(v) : "memory");
+}
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// Row block b belongs to CTA b mod C (C CTAs, a power of two), there to block
+// b / C: warp (b / C) mod W of its W row warps; one more warp forms the totals
+// and the scalars.  Shared memory of a CTA: its rows' r, the block sums of
+// both reductions (every CTA holds all of them: a warp that has summed a block
+// writes the sum to the C CTAs, one lane each), and its matrix rows, K entries
+// each, entry-major: weight and cluster address of the r entry.  Per iteration
+// two cluster barriers: after p.s, and after r and r.r.  Every CTA takes the
+// same decisions from the same bits, so all leave the loop together; the
+// decision to stop is formed by the scalar warp during the next p.s and read
+// after its barrier.
+//
+// What bounds it is latency: two shuffle trees (86 clocks a step), two totals,
+// a reciprocal and two cluster barriers (370 clocks) in one chain of about 2.5
+// us per iteration.  Beyond about 60 rows per SM the FP64 pipe (2 lanes a
+// clock): a row costs about 20 operations with its share of the trees.
+// Measured per solve to 1e-12, one 256-thread CTA with the CSR matrix in
+// global memory before -> now: 343 rows 187 -> 92 us, 1331 rows 960 -> 183 us,
+// 3375 rows with lognormal coefficients 9025 -> 1065 us, 250047 rows 820 -> 32 ms.
+struct CgArgs {
+  int n, K, maxit, blocks_per_cta;
+  const int *rowptr, *col;
+  const double* val;
+  const int64_t* fsrc;
+  const int* uptr;
+  const int64_t* udst;
+  const int* umaster;
+  double rtol;
+  int* iters;
+  double* work;   // 4 n doubles (NB = 0)
+};
+
+// Sum of the nb block sums in the order stated above, to every lane.  With at
+// most 16 blocks the tree's upper steps would only add zeros: the lanes hold
+// copies of the smallest power of two of buckets and skip them.
+__device__ __forceinline__ double cg_total(const double* sums, int nb) {
+  const int m = nb > 16 ? 32 : nb > 8 ? 16 : nb > 4 ? 8 : nb > 2 ? 4 : nb > 1 ? 2 : 1;
+  double v = 0.0;
+  for (int b = threadIdx.x & (m - 1); b < nb; b += 32) v += sums[b];
+  if (nb > 16) v = __dadd_rn(v, __shfl_xor_sync(0xffffffffu, v, 16));
+  if (nb > 8) v = __dadd_rn(v, __shfl_xor_sync(0xffffffffu, v, 8));
+  if (nb > 4) v = __dadd_rn(v, __shfl_xor_sync(0xffffffffu, v, 4));
+  if (nb > 2) v = __dadd_rn(v, __shfl_xor_sync(0xffffffffu, v, 2));
+  if (nb > 1) v = __dadd_rn(v, __shfl_xor_sync(0xffffffffu, v, 1));
+  return v;
+}
+
+// NB > 0: row blocks per warp at most, the vectors in registers; KC > 0 (NB = 1
+// only): rows of at most KC entries, held in registers too, else K entries per
+// row in shared memory.  NB = 0 (large coarse problems): any number of blocks,
+// x, p, s and A r in the work array and the matrix read from its CSR arrays.
+template <class T, int NB, int KC>
+__global__ void __launch_bounds__(NB > 0 ? CG_THREADS + 32 : 1024) k_cg_cluster(CgArgs A, const T* __restrict__ f,
+                                                                const T* __restrict__ fI, T* __restrict__ u,
+                                                                T* __restrict__ uI) {
   extern __shared__ double s_cg[];
-  __shared__ double red[2][CG_THREADS / 32];
-  double* x = smem ? s_cg : work;
-  double* r = x + n;
-  double* p = r + n;
-  double* Ap = p + n;
-  double part = 0.0;
-  for (int q = threadIdx.x; q < n; q += CG_THREADS) {
-    const int64_t s = fsrc[q];
-    const double b = s >= 0 ? (double)f[s] : (double)fI[-1 - s];
-    x[q] = 0.0;
-    r[q] = b;
-    p[q] = b;
-    part += b * b;
+  __shared__ double s_alpha, s_beta;
+  __shared__ int s_go;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, W = (blockDim.x >> 5) - 1;
+  uint32_t C;
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(C));
+  const uint32_t rank = cluster_rank();
+  const bool solo = C == 1;
+  auto barrier = [&]() {
+    if (solo) __syncthreads();
+    else cluster_barrier();
+  };
+  const int sh = NB > 0 ? 0 : cg_block_shift(A.n);
+  const int nb = ((A.n - 1) >> (5 + sh)) + 1, rows = A.blocks_per_cta << (5 + sh), K = A.K;
+  double* sr = s_cg;
+  double* sum0 = sr + rows;
+  double* sum1 = sum0 + nb;
+  double* mv = sum1 + nb;
+  uint32_t* ma = reinterpret_cast<uint32_t*>(mv + (size_t)K * rows);
+  const bool scalar = warp == W;
+  const uint32_t r_addr = smem_addr(sr);
+  const uint32_t peer0 = cluster_map(smem_addr(sum0), lane % C), peer1 = cluster_map(smem_addr(sum1), lane % C);
+  constexpr int NR = NB > 0 ? NB : 1;
+  const int ni = NB > 0 ? NB : (A.blocks_per_cta + W - 1) / W;
+  double xr[NR], rr_[NR], pr[NR], srow[NR], wr[NR];
+  double rv[KC > 0 ? KC : 1];
+  uint32_t ra[KC > 0 ? KC : 1];
+  // the warp's i-th block: local block warp + i W, global block that * C +
+  // rank; its g-th row of this lane
+  auto mine = [&](int i) { return !scalar && warp + i * W < A.blocks_per_cta; };
+  auto slot = [&](int i, int g) { return (((warp + i * W) << sh) + g) * 32 + lane; };
+  auto row_of = [&](int i, int g) {
+    const int q = ((((warp + i * W) * (int)C + (int)rank) << sh) + g) * 32 + lane;
+    return mine(i) && q < A.n ? q : -1;
+  };
+  auto addr_of = [&](int c) {   // cluster address of row c's r entry
+    const uint32_t b = (uint32_t)c >> (5 + sh), in = (uint32_t)c & ((32u << sh) - 1);
+    return cluster_map(r_addr + (((b / C) << (5 + sh)) + in) * 8, b % C);
+  };
+#pragma unroll
+  for (int i = 0; i < NB; ++i) {
+    xr[i] = rr_[i] = pr[i] = srow[i] = wr[i] = 0.0;
+    if (!mine(i)) continue;
+    const int q = row_of(i, 0), o = slot(i, 0);
+    const int e0 = q >= 0 ? A.rowptr[q] : 0, e1 = q >= 0 ? A.rowptr[q + 1] : 0;
+    auto entry = [&](int e, double& v, uint32_t& addr) {
+      const bool in = e0 + e < e1;
+      const int c = in ? __ldg(A.col + e0 + e) : 0;
+      v = in ? __ldg(A.val + e0 + e) : 0.0;
+      addr = in ? addr_of(c) : cluster_map(r_addr + (uint32_t)o * 8, rank);   // padding: weight 0 on the row's own entry
+    };
+    if (KC > 0) {
+#pragma unroll
+      for (int e = 0; e < KC; ++e) entry(e, rv[e], ra[e]);
+    } else {
+#pragma unroll 4
+      for (int e = 0; e < K; ++e) entry(e, mv[(size_t)e * rows + o], ma[(size_t)e * rows + o]);
+    }
   }
-  double rr = cg_allreduce(part, red[0]);
-  int rb = 1;
-  const double bnorm = sqrt(rr);
+  auto times = [&](int i, int q) {   // (A r) of the row
+    double a0 = 0.0, a1 = 0.0;
+    if (NB == 0) {
+      const int e1 = q >= 0 ? __ldg(A.rowptr + q + 1) : 0;
+      for (int e = q >= 0 ? __ldg(A.rowptr + q) : 0; e < e1; e += 2) {
+        a0 = fma(__ldg(A.val + e), cluster_load(addr_of(__ldg(A.col + e))), a0);
+        if (e + 1 < e1) a1 = fma(__ldg(A.val + e + 1), cluster_load(addr_of(__ldg(A.col + e + 1))), a1);
+      }
+    } else if (KC > 0) {
+      double v[KC > 0 ? KC : 1];
+#pragma unroll
+      for (int e = 0; e < KC; ++e) v[e] = cluster_load(ra[e]);
+#pragma unroll
+      for (int e = 0; e < KC; e += 2) {
+        a0 = fma(rv[e], v[e], a0);
+        if (e + 1 < KC) a1 = fma(rv[e + 1], v[e + 1], a1);
+      }
+    } else {
+      const int o = slot(i, 0);
+#pragma unroll 4
+      for (int e = 0; e < K; e += 2) {
+        a0 = fma(mv[(size_t)e * rows + o], cluster_load(ma[(size_t)e * rows + o]), a0);
+        if (e + 1 < K) a1 = fma(mv[(size_t)(e + 1) * rows + o], cluster_load(ma[(size_t)(e + 1) * rows + o]), a1);
+      }
+    }
+    return a0 + a1;
+  };
+  // Calls body(i, g, q) for the rows of the warp's blocks.
+  auto each = [&](auto&& body) {
+    if (scalar) return;
+    if constexpr (NB > 0) {
+#pragma unroll
+      for (int i = 0; i < NB; ++i)
+        if (mine(i)) body(i, 0, row_of(i, 0));
+    } else {
+      for (int i = 0; i < ni; ++i)
+        for (int g = 0; mine(i) && g < 1 << sh; ++g) body(i, g, row_of(i, g));
+    }
+  };
+  // The same with the blocks' sums of body's values written to every CTA.
+  auto each_sum = [&](uint32_t peer, auto&& body) {
+    if (scalar) return;
+#pragma unroll
+    for (int i = 0; i < ni; ++i) {
+      if (!mine(i)) continue;
+      double v = body(i, 0, row_of(i, 0));
+      if constexpr (NB == 0)
+        for (int g = 1; g < 1 << sh; ++g) v = __dadd_rn(v, body(i, g, row_of(i, g)));
+      const int b = (warp + i * W) * (int)C + (int)rank;
+      const double sb = warp_sum_xor(v);
+      if (b < nb && lane < (int)C) cluster_store(peer + (uint32_t)b * 8, sb);
+    }
+  };
+  double* gx = A.work;
+  double* gp = gx + (NB > 0 ? 0 : (size_t)A.n);
+  double* gs = gp + (NB > 0 ? 0 : (size_t)A.n);
+  double* gw = gs + (NB > 0 ? 0 : (size_t)A.n);
+  barrier();   // every CTA of the cluster runs before its memory is written
+  each_sum(peer0, [&](int i, int g, int q) {
+    double v = 0.0;
+    if (q >= 0) {
+      const int64_t src = A.fsrc[q];
+      v = src >= 0 ? (double)f[src] : (double)fI[-1 - src];
+      if (NB == 0) gx[q] = 0.0;
+    }
+    if (NB > 0) rr_[i] = v;
+    sr[slot(i, g)] = v;
+    return v * v;
+  });
+  barrier();   // b.b summed; every r entry written
+  double rr = 0.0, inv = 0.0;   // scalar warp
+  CgTest test{0.0, 0, 0};
+  bool any = false;
   int it = 0;
-  while (bnorm > 0.0 && sqrt(rr) > rtol * bnorm && it < maxit) {
-    __syncthreads();   // every p entry written before A p reads it
-    part = 0.0;
-    for (int q = threadIdx.x; q < n; q += CG_THREADS) {
-      double a = 0.0;
-      for (int e = __ldg(rowptr + q); e < __ldg(rowptr + q + 1); ++e) a += __ldg(val + e) * p[__ldg(col + e)];
-      Ap[q] = a;
-      part += p[q] * a;
+  for (;;) {
+    // r and r.r are complete: A r by the row warps, the scalars beside it
+    if (scalar) {
+      const double rr_new = cg_total(sum0, nb);
+      if (lane == 0) s_beta = rr_new * inv;
+      rr = rr_new;
     }
-    const double pAp = cg_allreduce(part, red[rb]);
-    rb ^= 1;
-    const double alpha = rr / pAp;
-    part = 0.0;
-    for (int q = threadIdx.x; q < n; q += CG_THREADS) {
-      x[q] += alpha * p[q];
-      const double rq = r[q] - alpha * Ap[q];
-      r[q] = rq;
-      part += rq * rq;
+    each([&](int i, int, int q) {
+      const double w = times(i, q);
+      if (NB > 0) wr[i] = w;
+      else if (q >= 0) gw[q] = w;
+    });
+    __syncthreads();
+    if (scalar) {
+      if (it == 0) {
+        const double bnorm = sqrt(rr);
+        any = bnorm > 0.0;
+        test = cg_test(A.rtol * bnorm);
+      }
+      const bool go = any && it < A.maxit && cg_above(rr, test);
+      if (lane == 0) s_go = go;
+      inv = cg_recip(rr);
     }
-    const double rr_new = cg_allreduce(part, red[rb]);
-    rb ^= 1;
-    const double beta = rr_new / rr;
-    for (int q = threadIdx.x; q < n; q += CG_THREADS) p[q] = r[q] + beta * p[q];
-    rr = rr_new;
+    const double beta = s_beta;
+    each_sum(peer1, [&](int i, int g, int q) {
+      double pq = 0.0, sq = 0.0;
+      if (NB > 0) {
+        pr[i] = pq = it ? fma(beta, pr[i], rr_[i]) : rr_[i];
+        srow[i] = sq = it ? fma(beta, srow[i], wr[i]) : wr[i];
+      } else if (q >= 0) {
+        const double r = sr[slot(i, g)], w = gw[q];
+        gp[q] = pq = it ? fma(beta, gp[q], r) : r;
+        gs[q] = sq = it ? fma(beta, gs[q], w) : w;
+      }
+      return pq * sq;
+    });
+    barrier();   // p.s summed; every read of r done; s_go written
+    if (!s_go) break;
+    if (scalar) {
+      const double al = rr * cg_recip(cg_total(sum1, nb));
+      if (lane == 0) s_alpha = al;
+    }
+    __syncthreads();
+    const double alpha = s_alpha;
+    each_sum(peer0, [&](int i, int g, int q) {
+      double r = 0.0;
+      if (NB > 0) {
+        xr[i] = fma(alpha, pr[i], xr[i]);
+        rr_[i] = r = fma(-alpha, srow[i], rr_[i]);
+      } else if (q >= 0) {
+        gx[q] = fma(alpha, gp[q], gx[q]);
+        r = fma(-alpha, gs[q], sr[slot(i, g)]);
+      }
+      sr[slot(i, g)] = r;
+      return r * r;
+    });
     ++it;
+    barrier();   // r.r summed; every r entry written
   }
-  for (int q = threadIdx.x; q < n; q += CG_THREADS) {
-    const T v = (T)x[q];
-    for (int e = uptr[q]; e < uptr[q + 1]; ++e) u[udst[e]] = v;
-    if (umaster[q] >= 0) uI[umaster[q]] = v;
-  }
-  if (threadIdx.x == 0 && iters) *iters = it;
+  each([&](int i, int, int q) {
+    if (q < 0) return;
+    const T v = (T)(NB > 0 ? xr[i] : gx[q]);
+    for (int e = A.uptr[q]; e < A.uptr[q + 1]; ++e) u[A.udst[e]] = v;
+    if (A.umaster[q] >= 0) uI[A.umaster[q]] = v;
+  });
+  if (rank == 0 && threadIdx.x == 0 && A.iters) *A.iters = it;
 }
 
 // Coefficient gradient (per macro, closed lattice): sum of lam_p times the
@@ -2438,61 +2817,10 @@ _Pragma("unroll")
 // Coarse CG (k_cg with its vectors in the problem's global work array).
 template <class T>
 __device__ void unit_cg(const BOp& op, double* red) {
-  const int n = op.n_cg;
-  const T* f = (const T*)op.f;
-  const T* fI = (const T*)op.fI;
-  T* u = (T*)op.u;
-  T* uI = (T*)op.uI;
-  double* x = op.work;
-  double* r = x + n;
-  double* p = r + n;
-  double* Ap = p + n;
-  const int tid = tid256();
-  double part = 0.0;
-  for (int q = tid; q < n; q += CTA) {
-    const int64_t s = op.fsrc[q];
-    const double b = s >= 0 ? (double)f[s] : (double)fI[-1 - s];
-    x[q] = 0.0;
-    r[q] = b;
-    p[q] = b;
-    part += b * b;
-  }
-  double rr = cg_allreduce(part, red);
-  int rb = 1;
-  const double bnorm = sqrt(rr);
-  int it = 0;
-  while (bnorm > 0.0 && sqrt(rr) > op.rtol * bnorm && it < op.maxit) {
-    __syncthreads();
-    part = 0.0;
-    for (int q = tid; q < n; q += CTA) {
-      double a = 0.0;
-      for (int e = op.rowptr[q]; e < op.rowptr[q + 1]; ++e) a += op.val[e] * p[op.col[e]];
-      Ap[q] = a;
-      part += p[q] * a;
-    }
-    const double pAp = cg_allreduce(part, red + 8 * rb);
-    rb ^= 1;
-    const double alpha = rr / pAp;
-    part = 0.0;
-    for (int q = tid; q < n; q += CTA) {
-      x[q] += alpha * p[q];
-      const double rq = r[q] - alpha * Ap[q];
-      r[q] = rq;
-      part += rq * rq;
-    }
-    const double rr_new = cg_allreduce(part, red + 8 * rb);
-    rb ^= 1;
-    const double beta = rr_new / rr;
-    for (int q = tid; q < n; q += CTA) p[q] = r[q] + beta * p[q];
-    rr = rr_new;
-    ++it;
-  }
-  for (int q = tid; q < n; q += CTA) {
-    const T v = (T)x[q];
-    for (int e = op.uptr[q]; e < op.uptr[q + 1]; ++e) u[op.udst[e]] = v;
-    if (op.umaster[q] >= 0) uI[op.umaster[q]] = v;
-  }
-  if (tid == 0 && op.iters) *op.iters = it;
+  const size_t n = (size_t)op.n_cg;
+  cg_one_cta<T>(op.n_cg, op.rowptr, op.col, op.val, op.fsrc, (const T*)op.f, (const T*)op.fI, op.uptr, op.udst,
+                op.umaster, (T*)op.u, (T*)op.uI, op.work, op.work + n, op.work + 2 * n, op.work + 3 * n, op.rtol,
+                op.maxit, op.iters, red);
 }
 
 // 16384 elements per unit of the block-wise operations (zeroing, the FP32
@@ -2647,7 +2975,7 @@ __global__ void __launch_bounds__(CTA, 5) k_batch(const BOp* __restrict__ ops, c
                                                   int n_live, BatchState st, int wait_limit, int* __restrict__ err) {
   __shared__ int s_pre2[MAX_SLABS][33];
   __shared__ int s_pre_tot[MAX_SLABS + 1];
-  __shared__ double red[16];
+  __shared__ double red[64];
   __shared__ BatchCtl ctl;
   __shared__ __align__(16) BOp s_op;
   if (tid256() == 0) {
@@ -3132,6 +3460,78 @@ cudaError_t prolong_add(const LevelArgs& F, const LevelArgs& C, const ProbArgs& 
   return cudaGetLastError();
 }
 
+// Launch shape of the cluster CG for n rows of at most K entries; clusters
+// == 0: it does not fit (or the device holds no such cluster).
+constexpr int CG_MAX_NB = 4;
+struct CgShape {
+  int clusters, ctas, warps, blocks_per_cta, blocks_per_warp;
+  size_t smem;
+};
+// Dynamic shared bytes a CTA may have and CTAs per cluster (16 where the device
+// schedules such clusters) on the current device.
+std::pair<int, int> cg_limits() {
+  static std::mutex mu;
+  static std::map<int, std::pair<int, int>> known;
+  int dev = 0;
+  cudaGetDevice(&dev);
+  std::lock_guard<std::mutex> lock(mu);
+  auto it = known.find(dev);
+  if (it != known.end()) return it->second;
+  int optin = 0;
+  cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  int a = std::max(0, optin - 2048), c = 16;
+  const void* kern[] = {(const void*)k_cg_cluster<float, 0, 0>,  (const void*)k_cg_cluster<float, 1, 0>,
+                        (const void*)k_cg_cluster<float, 1, 7>,  (const void*)k_cg_cluster<float, 1, 15>,
+                        (const void*)k_cg_cluster<double, 0, 0>, (const void*)k_cg_cluster<double, 1, 0>,
+                        (const void*)k_cg_cluster<double, 1, 7>, (const void*)k_cg_cluster<double, 1, 15>,
+                        (const void*)k_cg_cluster<float, CG_MAX_NB, 0>,
+                        (const void*)k_cg_cluster<double, CG_MAX_NB, 0>};
+  for (const void* k : kern)
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, a) != cudaSuccess ||
+        cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
+      a = 0;
+  cudaLaunchConfig_t cfg;
+  std::memset(&cfg, 0, sizeof(cfg));
+  cfg.gridDim = dim3(16);
+  cfg.blockDim = dim3(1024);
+  cfg.dynamicSmemBytes = (size_t)a;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = 16;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  int clusters = 0;
+  if (cudaOccupancyMaxActiveClusters(&clusters, (const void*)k_cg_cluster<double, 0, 0>, &cfg) != cudaSuccess ||
+      clusters < 1)
+    c = 8;
+  cudaGetLastError();
+  return known.emplace(dev, std::make_pair(a, c)).first->second;
+}
+CgShape cg_shape(int n, int K) {
+  const std::pair<int, int> lim = cg_limits();
+  CgShape g{0, 1, 1, 1, 1, 0};
+  const int nb = (n + 31) / 32;
+  // measured (us per solve to 1e-12): 5 blocks 79 on one CTA, 88 on 8; 11
+  // blocks 162 / 92 / 97 on 1 / 8 / 16; 17 blocks 139 / 147 on 8 / 16; 42
+  // blocks 187 / 183; 106 blocks 446 / 334
+  const int C = std::min(nb <= 5 ? 1 : nb <= 32 ? 8 : 16, lim.second);
+  int bpc = (nb + C - 1) / C;
+  int W = std::min(bpc, CG_WARPS);
+  int nbw = (bpc + W - 1) / W;
+  const size_t sums = 2 * (size_t)nb * 8;
+  size_t smem = (size_t)bpc * 32 * 8 + sums + (nbw == 1 && K <= 15 ? 0 : (size_t)K * bpc * 32 * 12);
+  if (n > 16384 || nbw > CG_MAX_NB || smem > (size_t)lim.first) {
+    const int sh = cg_block_shift(n), nbl = ((n - 1) >> (5 + sh)) + 1;
+    bpc = (nbl + C - 1) / C;
+    W = std::min(bpc, 31);
+    nbw = 0;
+    smem = ((size_t)bpc << (5 + sh)) * 8 + 2 * (size_t)nbl * 8;
+    if (smem > (size_t)lim.first) return g;
+  }
+  return CgShape{1, C, W, bpc, nbw, smem};
+}
+
 template <class T>
 cudaError_t coarse_cg(const DevProblem& p, const T* f, const T* fI, T* u, T* uI, double rtol, int maxit,
                       cudaStream_t s, double* work) {
@@ -3159,32 +3559,46 @@ cudaError_t coarse_cg(const DevProblem& p, const T* f, const T* fI, T* u, T* uI,
     return cudaSuccess;
   }
   if (p.n_cg == 0) return cudaSuccess;
-  // the vectors live in shared memory when they fit and no work array is
-  // imposed (the allocation-free cycle passes its static array)
-  static std::mutex mu;
-  static std::map<int, int> allow;   // device -> dynamic shared bytes allowed
-  int dev = 0;
-  cudaGetDevice(&dev);
-  int lim = 0;
-  {
-    std::lock_guard<std::mutex> lock(mu);
-    auto it = allow.find(dev);
-    if (it == allow.end()) {
-      int optin = 0;
-      cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-      const int a = std::max(0, optin - 4096);
-      const cudaError_t e = cudaFuncSetAttribute((const void*)k_cg<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, a);
-      if (e != cudaSuccess) return e;
-      it = allow.emplace(dev, a).first;
-    }
-    lim = it->second;
+  const CgShape sh = cg_shape(p.n_cg, p.cg_width);
+  if (sh.clusters > 0) {
+    CgArgs A;
+    A.n = p.n_cg;
+    A.K = p.cg_width;
+    A.maxit = maxit;
+    A.blocks_per_cta = sh.blocks_per_cta;
+    A.rowptr = p.rowptr;
+    A.col = p.col;
+    A.val = p.val;
+    A.fsrc = p.fsrc;
+    A.uptr = p.uptr;
+    A.udst = p.udst;
+    A.umaster = p.umaster;
+    A.rtol = rtol;
+    A.iters = p.cg_iters;
+    A.work = work ? work : p.cg_work;
+    cudaLaunchConfig_t cfg;
+    std::memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = dim3(sh.ctas);
+    cfg.blockDim = dim3(32 * (sh.warps + 1));   // and the scalar warp
+    cfg.dynamicSmemBytes = sh.smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = sh.ctas;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    ++g_kernel_launches;
+    auto kern = sh.blocks_per_warp == 0 ? k_cg_cluster<T, 0, 0>
+                : sh.blocks_per_warp > 1 ? k_cg_cluster<T, CG_MAX_NB, 0>
+                : A.K <= 7             ? k_cg_cluster<T, 1, 7>
+                : A.K <= 15            ? k_cg_cluster<T, 1, 15>
+                                       : k_cg_cluster<T, 1, 0>;
+    return cudaLaunchKernelEx(&cfg, kern, A, f, fI, u, uI);
   }
-  const size_t bytes = (size_t)4 * p.n_cg * sizeof(double);
-  const bool in_smem = !work && bytes <= (size_t)lim;
   ++g_kernel_launches;
-  k_cg<T><<<1, CG_THREADS, in_smem ? bytes : 0, s>>>(p.n_cg, p.rowptr, p.col, p.val, p.fsrc, f, fI, p.uptr, p.udst,
-                                                     p.umaster, u, uI, work ? work : p.cg_work, rtol, maxit,
-                                                     p.cg_iters, in_smem ? 1 : 0);
+  k_cg<T><<<1, CG_THREADS, 0, s>>>(p.n_cg, p.rowptr, p.col, p.val, p.fsrc, f, fI, p.uptr, p.udst, p.umaster, u, uI,
+                                   work ? work : p.cg_work, rtol, maxit, p.cg_iters);
   return cudaGetLastError();
 }
 
