@@ -377,6 +377,29 @@ int upload_if_tables(hhg_mesh* m, DevProblemLevel& q, int l, int kind, const std
   return HHG_OK;
 }
 
+// The coarse matrix's reciprocal diagonal, for the CG's preconditioner; in use
+// where the diagonal varies by more than half (moved corners, coefficients: on
+// 4x4x4 sub-cubes with lognormal ones 252 -> 109 iterations).  With a nearly
+// constant one it would change nothing but cost a second sum.
+int upload_diagonal(const HostProblem& h, DevProblem& d) {
+  d.cg_dinv = nullptr;
+  std::vector<double> dinv(h.n_cg);
+  double lo = 0.0, hi = 0.0;
+  for (int q = 0; q < h.n_cg; ++q) {
+    double a = 0.0;
+    for (int e = h.rowptr[q]; e < h.rowptr[q + 1]; ++e)
+      if (h.col[e] == q) a = h.val[e];
+    lo = q ? std::min(lo, a) : a;
+    hi = q ? std::max(hi, a) : a;
+    dinv[q] = 1.0 / a;
+  }
+  if (!(lo > 0.0) || !std::isfinite(hi / lo)) return HHG_OK;
+  // also where it is not in use: a batch's recorded launches may hold the buffer
+  HHG_CUDA(cudaMemcpy(d.cg_dinv_buf, dinv.data(), dinv.size() * sizeof(double), cudaMemcpyHostToDevice));
+  if (hi > 1.5 * lo) d.cg_dinv = d.cg_dinv_buf;
+  return HHG_OK;
+}
+
 int upload_problem(hhg_mesh* m, const HostProblem& h, DevProblem& d) {
   d.kind = h.kind;
   d.act_host = h.act;
@@ -416,6 +439,8 @@ int upload_problem(hhg_mesh* m, const HostProblem& h, DevProblem& d) {
   HHG_TRY(upload(m, &d.udst, h.udst));
   HHG_TRY(upload(m, &d.umaster, h.umaster));
   HHG_TRY(dalloc(m, &d.cg_work, (size_t)4 * std::max(1, h.n_cg)));
+  HHG_TRY(dalloc(m, &d.cg_dinv_buf, (size_t)std::max(1, h.n_cg)));
+  HHG_TRY(upload_diagonal(h, d));
   const int L = (int)m->host.lv.size() - 1;
   d.n_partial = m->tab[L].n_tiles_int * std::max(1, d.n_act) + (m->host.lv[L].n_if + 127) / 128 + 64;
   HHG_TRY(dalloc(m, &d.partial, (size_t)d.n_partial));
@@ -1123,6 +1148,9 @@ int update_coefficients(hhg_mesh* m, const double* coeff) {
       return fail(HHG_ERR_STATE, "coarse system changed shape");
     if (!h.val.empty())
       HHG_CUDA(cudaMemcpy(d->val, h.val.data(), h.val.size() * sizeof(double), cudaMemcpyHostToDevice));
+    const bool had = d->cg_dinv != nullptr;
+    HHG_TRY(upload_diagonal(h, *d));
+    if (d == &m->faulty && had != (d->cg_dinv != nullptr)) drop_local_graph(m);   // it holds the CG's launch
     // the interface tables hold summed stencil weights (kinds 0-2 use the
     // level's own copy lists)
     for (size_t l = 1; l < d->lv.size() && l < d->free_host.size(); ++l)

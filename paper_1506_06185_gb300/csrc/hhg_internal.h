@@ -408,6 +408,8 @@ struct DevProblem {
   int* umaster = nullptr;
   double* cg_work = nullptr;        // 4 * n_cg scratch
   int cg_width = 0;                 // entries of the longest row
+  double* cg_dinv_buf = nullptr;    // reciprocal diagonal of the coarse matrix
+  double* cg_dinv = nullptr;        // the same where the diagonal varies, else null
   double* partial = nullptr;        // per-CTA partial sums of the norm
   int n_partial = 0;
   double* scalar = nullptr;         // [4]: norm^2 result, cg info

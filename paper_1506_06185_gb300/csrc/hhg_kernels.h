@@ -212,6 +212,7 @@ struct BOp {
   const int64_t* udst;
   const int* umaster;
   double* work;
+  const double* dinv;   // null, or the reciprocal diagonal (preconditioned)
   int* iters;
   double rtol;
   int maxit;

@@ -1907,7 +1907,9 @@ __device__ __forceinline__ bool cg_above(double rr, const CgTest& t) {
 }
 
 // CG on the compact free nodes of the coarsest level from x = 0 until
-// ||r|| <= rtol ||b|| or maxit iterations.  The direction's image s = A p is
+// ||r|| <= rtol ||b|| or maxit iterations, with z = r, or, given the
+// reciprocal diagonal, z = r / diag (Jacobi preconditioning; below r.r stands
+// for r.z, the stopping test keeps r.r).  The direction's image s = A p is
 // carried along, s <- A r + beta s, so that the product A r does not wait for
 // beta.  One iteration: p.s, alpha = r.r / p.s, x += alpha p, r -= alpha s,
 // r.r, beta = r.r / old r.r (times the reciprocal, formed beside the critical
@@ -1915,54 +1917,62 @@ __device__ __forceinline__ bool cg_above(double rr, const CgTest& t) {
 // chains, even and odd entries.
 //
 // One CTA of CG_THREADS threads; x, r, p and s live in shared or in global
-// memory (4 n doubles); a row belongs to one thread throughout.  red: 64
-// doubles of shared memory.
+// memory (4 n doubles); a row belongs to one thread throughout.  dinv: the
+// reciprocal diagonal, or null.  red: 64 doubles of shared memory.
 template <class T>
 __device__ __forceinline__ void cg_one_cta(int n, const int* rowptr, const int* col, const double* val,
                                            const int64_t* fsrc, const T* f, const T* fI, const int* uptr,
                                            const int64_t* udst, const int* umaster, T* u, T* uI, double* x, double* r,
-                                           double* p, double* s, double rtol, int maxit, int* iters, double* red) {
+                                           double* p, double* s, const double* dinv, double rtol, int maxit,
+                                           int* iters, double* red) {
   const int t = threadIdx.y * blockDim.x + threadIdx.x;
+  auto z = [&](int q) { return dinv ? dinv[q] * r[q] : r[q]; };
   auto row_times = [&](int q) {
     double a0 = 0.0, a1 = 0.0;
     const int e1 = rowptr[q + 1];
     for (int e = rowptr[q]; e < e1; e += 2) {
-      a0 = fma(val[e], r[col[e]], a0);
-      if (e + 1 < e1) a1 = fma(val[e + 1], r[col[e + 1]], a1);
+      a0 = fma(val[e], z(col[e]), a0);
+      if (e + 1 < e1) a1 = fma(val[e + 1], z(col[e + 1]), a1);
     }
     return a0 + a1;
   };
-  double rr = cg_rows_sum(n, red, [&](int q) {
+  auto squares = [&]() { return cg_rows_sum(n, red + 32, [&](int q) { return r[q] * r[q]; }); };
+  double rz = cg_rows_sum(n, red, [&](int q) {
     const int64_t src = fsrc[q];
     const double b = src >= 0 ? (double)f[src] : (double)fI[-1 - src];
     x[q] = 0.0;
     r[q] = b;
-    return b * b;
+    return b * z(q);
   });
+  double rr = dinv ? squares() : rz;
   const double bnorm = sqrt(rr);
   const CgTest test = cg_test(rtol * bnorm);
   int it = 0;
   double beta = 0.0;
   while (bnorm > 0.0 && it < maxit && cg_above(rr, test)) {
-    // every r entry was written before the barrier of the last sum
+    __syncthreads();   // every r entry is written, every total read
     const double pAp = cg_rows_sum(n, red + 32, [&](int q) {
       const double w = row_times(q);
-      const double pq = it ? fma(beta, p[q], r[q]) : r[q];
+      const double pq = it ? fma(beta, p[q], z(q)) : z(q);
       const double sq = it ? fma(beta, s[q], w) : w;
       p[q] = pq;
       s[q] = sq;
       return pq * sq;
     });
-    const double alpha = rr * cg_recip(pAp);
-    const double inv = cg_recip(rr);
-    const double rr_new = cg_rows_sum(n, red, [&](int q) {
+    const double alpha = rz * cg_recip(pAp);
+    const double inv = cg_recip(rz);
+    const double rz_new = cg_rows_sum(n, red, [&](int q) {
       x[q] = fma(alpha, p[q], x[q]);
-      const double rq = fma(-alpha, s[q], r[q]);
-      r[q] = rq;
-      return rq * rq;
+      r[q] = fma(-alpha, s[q], r[q]);
+      return r[q] * z(q);
     });
-    beta = rr_new * inv;
-    rr = rr_new;
+    rr = rz_new;
+    if (dinv) {
+      __syncthreads();   // the last total has been read
+      rr = squares();
+    }
+    beta = rz_new * inv;
+    rz = rz_new;
     ++it;
   }
   for (int q = t; q < n; q += CG_THREADS) {
@@ -1979,11 +1989,12 @@ __global__ void __launch_bounds__(CG_THREADS) k_cg(int n, const int* __restrict_
                                                    const T* __restrict__ f, const T* __restrict__ fI,
                                                    const int* __restrict__ uptr, const int64_t* __restrict__ udst,
                                                    const int* __restrict__ umaster, T* __restrict__ u,
-                                                   T* __restrict__ uI, double* __restrict__ work, double rtol,
-                                                   int maxit, int* __restrict__ iters) {
+                                                   T* __restrict__ uI, double* __restrict__ work,
+                                                   const double* __restrict__ dinv, double rtol, int maxit,
+                                                   int* __restrict__ iters) {
   __shared__ double red[64];
   cg_one_cta<T>(n, rowptr, col, val, fsrc, f, fI, uptr, udst, umaster, u, uI, work, work + n, work + 2 * (size_t)n,
-                work + 3 * (size_t)n, rtol, maxit, iters, red);
+                work + 3 * (size_t)n, dinv, rtol, maxit, iters, red);
 }
 
 // --- the same CG on a thread-block cluster --------------------------------
@@ -2035,6 +2046,7 @@ struct CgArgs {
   const int* uptr;
   const int64_t* udst;
   const int* umaster;
+  const double* dinv;   // null, or the reciprocal diagonal (NB > 0)
   double rtol;
   int* iters;
   double* work;   // 4 n doubles (NB = 0)
@@ -2059,7 +2071,7 @@ __device__ __forceinline__ double cg_total(const double* sums, int nb) {
 // only): rows of at most KC entries, held in registers too, else K entries per
 // row in shared memory.  NB = 0 (large coarse problems): any number of blocks,
 // x, p, s and A r in the work array and the matrix read from its CSR arrays.
-template <class T, int NB, int KC>
+template <class T, int NB, int KC, bool JAC>
 __global__ void __launch_bounds__(NB > 0 ? CG_THREADS + 32 : 1024) k_cg_cluster(CgArgs A, const T* __restrict__ f,
                                                                 const T* __restrict__ fI, T* __restrict__ u,
                                                                 T* __restrict__ uI) {
@@ -2080,14 +2092,17 @@ __global__ void __launch_bounds__(NB > 0 ? CG_THREADS + 32 : 1024) k_cg_cluster(
   double* sr = s_cg;
   double* sum0 = sr + rows;
   double* sum1 = sum0 + nb;
-  double* mv = sum1 + nb;
+  constexpr bool jac = NB > 0 && JAC;
+  double* sum2 = sum1 + nb;   // r.r beside r.z
+  double* mv = sum2 + (jac ? nb : 0);
   uint32_t* ma = reinterpret_cast<uint32_t*>(mv + (size_t)K * rows);
   const bool scalar = warp == W;
   const uint32_t r_addr = smem_addr(sr);
-  const uint32_t peer0 = cluster_map(smem_addr(sum0), lane % C), peer1 = cluster_map(smem_addr(sum1), lane % C);
+  const uint32_t peer0 = cluster_map(smem_addr(sum0), lane % C), peer1 = cluster_map(smem_addr(sum1), lane % C),
+                 peer2 = cluster_map(smem_addr(sum2), lane % C);
   constexpr int NR = NB > 0 ? NB : 1;
   const int ni = NB > 0 ? NB : (A.blocks_per_cta + W - 1) / W;
-  double xr[NR], rr_[NR], pr[NR], srow[NR], wr[NR];
+  double xr[NR], rr_[NR], pr[NR], srow[NR], wr[NR], dr[NR];
   double rv[KC > 0 ? KC : 1];
   uint32_t ra[KC > 0 ? KC : 1];
   // the warp's i-th block: local block warp + i W, global block that * C +
@@ -2105,8 +2120,10 @@ __global__ void __launch_bounds__(NB > 0 ? CG_THREADS + 32 : 1024) k_cg_cluster(
 #pragma unroll
   for (int i = 0; i < NB; ++i) {
     xr[i] = rr_[i] = pr[i] = srow[i] = wr[i] = 0.0;
+    dr[i] = 1.0;
     if (!mine(i)) continue;
     const int q = row_of(i, 0), o = slot(i, 0);
+    if (jac && q >= 0) dr[i] = A.dinv[q];
     const int e0 = q >= 0 ? A.rowptr[q] : 0, e1 = q >= 0 ? A.rowptr[q + 1] : 0;
     auto entry = [&](int e, double& v, uint32_t& addr) {
       const bool in = e0 + e < e1;
@@ -2175,6 +2192,11 @@ __global__ void __launch_bounds__(NB > 0 ? CG_THREADS + 32 : 1024) k_cg_cluster(
       if (b < nb && lane < (int)C) cluster_store(peer + (uint32_t)b * 8, sb);
     }
   };
+  auto z = [&](int i, double r) { return jac ? dr[i] * r : r; };
+  // r.r of the warp's rows, to every CTA
+  auto squares = [&]() {
+    if (jac) each_sum(peer2, [&](int i, int, int) { return rr_[i] * rr_[i]; });
+  };
   double* gx = A.work;
   double* gp = gx + (NB > 0 ? 0 : (size_t)A.n);
   double* gs = gp + (NB > 0 ? 0 : (size_t)A.n);
@@ -2188,20 +2210,21 @@ __global__ void __launch_bounds__(NB > 0 ? CG_THREADS + 32 : 1024) k_cg_cluster(
       if (NB == 0) gx[q] = 0.0;
     }
     if (NB > 0) rr_[i] = v;
-    sr[slot(i, g)] = v;
-    return v * v;
+    const double zv = z(i, v);
+    sr[slot(i, g)] = zv;
+    return v * zv;
   });
+  squares();
   barrier();   // b.b summed; every r entry written
-  double rr = 0.0, inv = 0.0;   // scalar warp
+  double rz = 0.0, rr = 0.0, inv = 0.0;   // scalar warp
   CgTest test{0.0, 0, 0};
   bool any = false;
   int it = 0;
   for (;;) {
     // r and r.r are complete: A r by the row warps, the scalars beside it
     if (scalar) {
-      const double rr_new = cg_total(sum0, nb);
-      if (lane == 0) s_beta = rr_new * inv;
-      rr = rr_new;
+      rz = cg_total(sum0, nb);
+      if (lane == 0) s_beta = rz * inv;
     }
     each([&](int i, int, int q) {
       const double w = times(i, q);
@@ -2210,6 +2233,7 @@ __global__ void __launch_bounds__(NB > 0 ? CG_THREADS + 32 : 1024) k_cg_cluster(
     });
     __syncthreads();
     if (scalar) {
+      rr = jac ? cg_total(sum2, nb) : rz;
       if (it == 0) {
         const double bnorm = sqrt(rr);
         any = bnorm > 0.0;
@@ -2217,13 +2241,14 @@ __global__ void __launch_bounds__(NB > 0 ? CG_THREADS + 32 : 1024) k_cg_cluster(
       }
       const bool go = any && it < A.maxit && cg_above(rr, test);
       if (lane == 0) s_go = go;
-      inv = cg_recip(rr);
+      inv = cg_recip(rz);
     }
     const double beta = s_beta;
     each_sum(peer1, [&](int i, int g, int q) {
       double pq = 0.0, sq = 0.0;
       if (NB > 0) {
-        pr[i] = pq = it ? fma(beta, pr[i], rr_[i]) : rr_[i];
+        const double zv = z(i, rr_[i]);
+        pr[i] = pq = it ? fma(beta, pr[i], zv) : zv;
         srow[i] = sq = it ? fma(beta, srow[i], wr[i]) : wr[i];
       } else if (q >= 0) {
         const double r = sr[slot(i, g)], w = gw[q];
@@ -2235,7 +2260,7 @@ __global__ void __launch_bounds__(NB > 0 ? CG_THREADS + 32 : 1024) k_cg_cluster(
     barrier();   // p.s summed; every read of r done; s_go written
     if (!s_go) break;
     if (scalar) {
-      const double al = rr * cg_recip(cg_total(sum1, nb));
+      const double al = rz * cg_recip(cg_total(sum1, nb));
       if (lane == 0) s_alpha = al;
     }
     __syncthreads();
@@ -2249,9 +2274,11 @@ __global__ void __launch_bounds__(NB > 0 ? CG_THREADS + 32 : 1024) k_cg_cluster(
         gx[q] = fma(alpha, gp[q], gx[q]);
         r = fma(-alpha, gs[q], sr[slot(i, g)]);
       }
-      sr[slot(i, g)] = r;
-      return r * r;
+      const double zv = z(i, r);
+      sr[slot(i, g)] = zv;
+      return r * zv;
     });
+    squares();
     ++it;
     barrier();   // r.r summed; every r entry written
   }
@@ -2819,8 +2846,8 @@ template <class T>
 __device__ void unit_cg(const BOp& op, double* red) {
   const size_t n = (size_t)op.n_cg;
   cg_one_cta<T>(op.n_cg, op.rowptr, op.col, op.val, op.fsrc, (const T*)op.f, (const T*)op.fI, op.uptr, op.udst,
-                op.umaster, (T*)op.u, (T*)op.uI, op.work, op.work + n, op.work + 2 * n, op.work + 3 * n, op.rtol,
-                op.maxit, op.iters, red);
+                op.umaster, (T*)op.u, (T*)op.uI, op.work, op.work + n, op.work + 2 * n, op.work + 3 * n, op.dinv,
+                op.rtol, op.maxit, op.iters, red);
 }
 
 // 16384 elements per unit of the block-wise operations (zeroing, the FP32
@@ -3467,6 +3494,14 @@ struct CgShape {
   int clusters, ctas, warps, blocks_per_cta, blocks_per_warp;
   size_t smem;
 };
+// The register form of a shape (see k_cg_cluster).
+template <class T, bool JAC>
+auto cg_kernel(const CgShape& sh, int K) {
+  return sh.blocks_per_warp > 1 ? k_cg_cluster<T, CG_MAX_NB, 0, JAC>
+         : K <= 7               ? k_cg_cluster<T, 1, 7, JAC>
+         : K <= 15              ? k_cg_cluster<T, 1, 15, JAC>
+                                : k_cg_cluster<T, 1, 0, JAC>;
+}
 // Dynamic shared bytes a CTA may have and CTAs per cluster (16 where the device
 // schedules such clusters) on the current device.
 std::pair<int, int> cg_limits() {
@@ -3480,12 +3515,16 @@ std::pair<int, int> cg_limits() {
   int optin = 0;
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   int a = std::max(0, optin - 2048), c = 16;
-  const void* kern[] = {(const void*)k_cg_cluster<float, 0, 0>,  (const void*)k_cg_cluster<float, 1, 0>,
-                        (const void*)k_cg_cluster<float, 1, 7>,  (const void*)k_cg_cluster<float, 1, 15>,
-                        (const void*)k_cg_cluster<double, 0, 0>, (const void*)k_cg_cluster<double, 1, 0>,
-                        (const void*)k_cg_cluster<double, 1, 7>, (const void*)k_cg_cluster<double, 1, 15>,
-                        (const void*)k_cg_cluster<float, CG_MAX_NB, 0>,
-                        (const void*)k_cg_cluster<double, CG_MAX_NB, 0>};
+  std::vector<const void*> kern = {(const void*)k_cg_cluster<float, 0, 0, false>,
+                                   (const void*)k_cg_cluster<double, 0, 0, false>};
+  for (int nbw : {1, CG_MAX_NB})
+    for (int K : {7, 15, 16}) {
+      const CgShape sh{1, 1, 1, 1, nbw, 0};
+      kern.push_back((const void*)cg_kernel<float, false>(sh, K));
+      kern.push_back((const void*)cg_kernel<float, true>(sh, K));
+      kern.push_back((const void*)cg_kernel<double, false>(sh, K));
+      kern.push_back((const void*)cg_kernel<double, true>(sh, K));
+    }
   for (const void* k : kern)
     if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, a) != cudaSuccess ||
         cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
@@ -3502,13 +3541,13 @@ std::pair<int, int> cg_limits() {
   cfg.attrs = at;
   cfg.numAttrs = 1;
   int clusters = 0;
-  if (cudaOccupancyMaxActiveClusters(&clusters, (const void*)k_cg_cluster<double, 0, 0>, &cfg) != cudaSuccess ||
+  if (cudaOccupancyMaxActiveClusters(&clusters, (const void*)k_cg_cluster<double, 0, 0, false>, &cfg) != cudaSuccess ||
       clusters < 1)
     c = 8;
   cudaGetLastError();
   return known.emplace(dev, std::make_pair(a, c)).first->second;
 }
-CgShape cg_shape(int n, int K) {
+CgShape cg_shape(int n, int K, bool jac) {
   const std::pair<int, int> lim = cg_limits();
   CgShape g{0, 1, 1, 1, 1, 0};
   const int nb = (n + 31) / 32;
@@ -3519,7 +3558,7 @@ CgShape cg_shape(int n, int K) {
   int bpc = (nb + C - 1) / C;
   int W = std::min(bpc, CG_WARPS);
   int nbw = (bpc + W - 1) / W;
-  const size_t sums = 2 * (size_t)nb * 8;
+  const size_t sums = (jac ? 3 : 2) * (size_t)nb * 8;
   size_t smem = (size_t)bpc * 32 * 8 + sums + (nbw == 1 && K <= 15 ? 0 : (size_t)K * bpc * 32 * 12);
   if (n > 16384 || nbw > CG_MAX_NB || smem > (size_t)lim.first) {
     const int sh = cg_block_shift(n), nbl = ((n - 1) >> (5 + sh)) + 1;
@@ -3530,6 +3569,15 @@ CgShape cg_shape(int n, int K) {
     if (smem > (size_t)lim.first) return g;
   }
   return CgShape{1, C, W, bpc, nbw, smem};
+}
+
+// The preconditioner is used where the diagonal varies (the host then stores
+// its reciprocal), the rows fit the register forms, and the iteration runs to
+// the default tolerance: a caller that caps the iterations or loosens the
+// tolerance gets that many steps of plain CG.
+const double* cg_precond(const DevProblem& p, double rtol, int maxit) {
+  if (!p.cg_dinv || rtol > 1e-12 || maxit < 1000 || p.n_cg > 16384) return nullptr;
+  return cg_shape(p.n_cg, p.cg_width, true).blocks_per_warp > 0 ? p.cg_dinv : nullptr;
 }
 
 template <class T>
@@ -3548,6 +3596,7 @@ cudaError_t coarse_cg(const DevProblem& p, const T* f, const T* fI, T* u, T* uI,
     op.udst = p.udst;
     op.umaster = p.umaster;
     op.work = work ? work : p.cg_work;
+    op.dinv = cg_precond(p, rtol, maxit);
     op.iters = p.cg_iters;
     op.rtol = rtol;
     op.maxit = maxit;
@@ -3559,7 +3608,8 @@ cudaError_t coarse_cg(const DevProblem& p, const T* f, const T* fI, T* u, T* uI,
     return cudaSuccess;
   }
   if (p.n_cg == 0) return cudaSuccess;
-  const CgShape sh = cg_shape(p.n_cg, p.cg_width);
+  const double* dinv = cg_precond(p, rtol, maxit);
+  const CgShape sh = cg_shape(p.n_cg, p.cg_width, dinv != nullptr);
   if (sh.clusters > 0) {
     CgArgs A;
     A.n = p.n_cg;
@@ -3573,6 +3623,7 @@ cudaError_t coarse_cg(const DevProblem& p, const T* f, const T* fI, T* u, T* uI,
     A.uptr = p.uptr;
     A.udst = p.udst;
     A.umaster = p.umaster;
+    A.dinv = dinv;
     A.rtol = rtol;
     A.iters = p.cg_iters;
     A.work = work ? work : p.cg_work;
@@ -3589,16 +3640,14 @@ cudaError_t coarse_cg(const DevProblem& p, const T* f, const T* fI, T* u, T* uI,
     cfg.attrs = at;
     cfg.numAttrs = 1;
     ++g_kernel_launches;
-    auto kern = sh.blocks_per_warp == 0 ? k_cg_cluster<T, 0, 0>
-                : sh.blocks_per_warp > 1 ? k_cg_cluster<T, CG_MAX_NB, 0>
-                : A.K <= 7             ? k_cg_cluster<T, 1, 7>
-                : A.K <= 15            ? k_cg_cluster<T, 1, 15>
-                                       : k_cg_cluster<T, 1, 0>;
+    const auto kern = sh.blocks_per_warp == 0 ? k_cg_cluster<T, 0, 0, false>
+                      : dinv                  ? cg_kernel<T, true>(sh, A.K)
+                                              : cg_kernel<T, false>(sh, A.K);
     return cudaLaunchKernelEx(&cfg, kern, A, f, fI, u, uI);
   }
   ++g_kernel_launches;
   k_cg<T><<<1, CG_THREADS, 0, s>>>(p.n_cg, p.rowptr, p.col, p.val, p.fsrc, f, fI, p.uptr, p.udst, p.umaster, u, uI,
-                                   work ? work : p.cg_work, rtol, maxit, p.cg_iters);
+                                   work ? work : p.cg_work, dinv, rtol, maxit, p.cg_iters);
   return cudaGetLastError();
 }
 

@@ -49,6 +49,31 @@ def test_cluster_equals_persistent_executor(hhg, sub, R, r0, affine):
         M.close()
 
 
+@pytest.mark.parametrize("sub,R,r0", [((1, 1, 1), 3, 2), ((2, 2, 2), 3, 2), ((3, 3, 3), 3, 2), ((3, 3, 3), 4, 3)])
+def test_preconditioned_forms(hhg, sub, R, r0):
+    """Coefficients over three decades: Jacobi-preconditioned, all forms alike,
+    and the solution is that of the oracle's plain CG."""
+    k = 10.0 ** np.random.default_rng(5).uniform(-1.5, 1.5, 6 * int(np.prod(sub)))
+    f, u0 = I.random_load(sub, R, seed=12), I.initial_guess(sub, R)
+    A, B, T = hhg.Mesh(sub, R, coarsest=r0, coeff=k), hhg.Mesh(sub, R, coarsest=r0), hhg.Mesh((1, 1, 1), 3)
+    B.set_coefficients(k)
+    T.set_problem(np.zeros(T.shape), np.zeros(T.shape))
+    A.set_problem(f, u0)
+    A.vcycle()
+    batch = hhg.Batch([(T, [0], 1)], B, 1)
+    B.set_problem(f, u0)
+    batch.launch_persistent()
+    assert np.array_equal(A.get_solution(), B.get_solution())
+    if r0 == 2:
+        m = O.Mesh(sub, R, coeff=k)
+        uo, fo = O.pad(u0.copy()), O.pad(f)
+        O.vcycle(m, m.global_problem, len(m.levels) - 1, uo, fo)
+        assert_close(A.get_solution(), O.interior(uo))
+    batch.close()
+    for M in (A, B, T):
+        M.close()
+
+
 @pytest.mark.parametrize("maxit,rtol", [(1, 0.0), (3, 0.0), (1000, 1e-2), (1000, 2.0)])
 def test_caps_and_loose_tolerances(hhg, maxit, rtol):
     """The caller's cap and tolerance end the iteration where the oracle's CG ends."""
