@@ -276,8 +276,8 @@ int hhg_grad_coeff(hhg_mesh* mesh, const double* u, const double* lam, double* g
  * the global problem with each candidate tile shape (nodes per tile and
  * slices per tile: 256/4, 512/8, 1024/8, 2048/16) on the FP64 iterate (which
  * the sweeps smooth) and, on precision-32 meshes, also on the FP32 arrays,
- * and keeps for that level the shape with the least total time; on meshes
- * with the 7-point structure it then times the flat Gauss-Seidel kernel
+ * and keeps for that level the shape with the least total time; it then
+ * times the flat Gauss-Seidel kernel
  * (hhg_set_flat_gs) and keeps it for the level's sweeps if it is faster
  * still (the residual and transfer kernels keep the chosen tiles).
  * chosen (may be NULL, one int per level, coarsest first) receives the index
@@ -437,14 +437,16 @@ int hhg_walk_counts(hhg_mesh* mesh, int64_t* counts);
  * with hhg_set_problem).  tries = 0 makes every wait run out at once, which
  * exercises that path without any fault. */
 int hhg_set_streaming(hhg_mesh* mesh, int enable);
-/* hhg_set_flat_gs: enable or disable (default) the flat Gauss-Seidel kernel on
- * every smoothed level of a mesh with the 7-point structure (ignored on
- * meshes without it; general connectivity: HHG_ERR_STATE; HHG_ERR_ARG, with
- * nothing changed, when a level has more than 1024 intervals per macro edge
- * or 2^31 items per launch): one thread per
- * 16-byte vector of same-colour nodes, indexed through a per-level item
+/* hhg_set_flat_gs: enable the flat kernels on every smoothed level of a mesh
+ * with the 7-point structure, or disable them there (ignored on meshes without
+ * it; general connectivity: HHG_ERR_STATE; HHG_ERR_ARG, with nothing changed,
+ * when a level has more than 1024 intervals per macro edge or 2^31 items per
+ * launch).  A new mesh of any stencil or connectivity has them on by default
+ * on every level that they can run, except while a launch limit
+ * (hhg_set_launch_limit) is set, which selects the tile kernels.  One thread
+ * per 16-byte vector of same-colour nodes, indexed through a per-level item
  * table (4 bytes per item, FP64 and on precision-32 meshes FP32 tables,
- * allocated on enable and freed on disable), with no tiles and no CTA
+ * allocated with the level and freed on disable), with no tiles and no CTA
  * barrier, which suits the small coarse levels; hhg_autotune picks it per
  * level.  On those levels the residual before each restriction, the
  * restriction onto the level (one thread per slot of four coarse nodes) and

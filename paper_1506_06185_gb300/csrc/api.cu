@@ -1166,9 +1166,6 @@ int update_coefficients(hhg_mesh* m, const double* coeff) {
 const int TUNE_CAND[][2] = {{256, 4}, {512, 8}, {1024, 8}, {2048, 16}};
 constexpr int N_TUNE_CAND = 4;
 
-// Flat Gauss-Seidel on level l (7-point meshes of the cube family): build and
-// upload its item tables (FP64, and FP32 on precision-32 meshes) when
-// switching it on, free them when switching it off.
 // Whether the flat kernels can run level l: 4 .. 1024 intervals per macro edge
 // (the packed items hold j, k and the group in 10 bits each) and every item
 // count times the macros below 2^31 (the kernels' thread indices are 32-bit;
@@ -1191,10 +1188,13 @@ bool flat_fits(const hhg_mesh* m, int l) {
   return std::max(items, slots) * m->host.n_macro <= limit;
 }
 
-int set_flat(hhg_mesh* m, int l, bool on) {
+// The flat kernels on level l: build and upload the item tables (FP64, and FP32
+// on precision-32 meshes, and the restriction's slots) when switching them on,
+// free them when switching them off.
+int set_flat(hhg_mesh* m, int l, int mode) {
   DevLevelTables& tb = m->tab[l];
   const HostLevel& H = m->host.lv[l];
-  if (!on) {
+  if (mode == FLAT_OFF) {
     std::vector<void*> unused;
     for (void* q : {(void*)tb.gs_items64, (void*)tb.gs_items32, (void*)tb.slot_items})
       if (q) unused.push_back(q);
@@ -1210,7 +1210,7 @@ int set_flat(hhg_mesh* m, int l, bool on) {
     return fail(HHG_ERR_ARG, "the flat kernels need 4 .. 1024 intervals per macro edge and fewer than 2^31 "
                              "items per launch");
   for (int vw : {2, 4}) {
-    if (vw == 4 && m->precision != 32) continue;
+    if (l == 0 || (vw == 4 && m->precision != 32)) continue;   // level 0 is not smoothed
     uint32_t*& dst = vw == 2 ? tb.gs_items64 : tb.gs_items32;
     if (dst) continue;
     std::vector<uint32_t> items;
@@ -1225,7 +1225,7 @@ int set_flat(hhg_mesh* m, int l, bool on) {
     HHG_TRY(upload(m, &tb.slot_items, slots));
     tb.n_slots = (int)slots.size();
   }
-  tb.gs_flat = 1;
+  tb.gs_flat = mode;
   return HHG_OK;
 }
 
@@ -1245,7 +1245,7 @@ int time_smooth(hhg_mesh* m, Prec<T>& P, int l, int reps, cudaStream_t s, cudaEv
 int tune_level(hhg_mesh* m, int l, int reps, cudaStream_t s, int* best_out) {
   const HostLevel& H = m->host.lv[l];
   DevLevelTables& tb = m->tab[l];
-  HHG_TRY(set_flat(m, l, false));   // the tile candidates are timed with the tile kernel
+  HHG_TRY(set_flat(m, l, FLAT_OFF));   // the tile candidates are timed with the tile kernel
   Tile* const before = tb.tiles_int;
   double best_ms = 1e30;
   int best = -1;
@@ -1275,15 +1275,15 @@ int tune_level(hhg_mesh* m, int l, int reps, cudaStream_t s, int* best_out) {
   tb.tiles_int = dev[best];
   tb.n_tiles_int = ndev[best];
   *best_out = best;
-  // the flat Gauss-Seidel kernel against the best tile shape (7-point
-  // levels); the level's other kernels keep the tiles either way
-  if (m->host.seven_point && flat_fits(m, l)) {
-    HHG_TRY(set_flat(m, l, true));
+  // the flat Gauss-Seidel kernel against the best tile shape; the level's
+  // other kernels keep the tiles either way
+  if (flat_fits(m, l)) {
+    HHG_TRY(set_flat(m, l, FLAT_ON));
     float ms = 0.f, ms32 = 0.f;
     HHG_TRY(time_smooth<double>(m, m->d64, l, reps, s, a, b, &ms));
     if (m->precision == 32) HHG_TRY(time_smooth<float>(m, m->d32, l, reps, s, a, b, &ms32));
     if (ms + ms32 < best_ms) *best_out = best + N_TUNE_CAND;
-    else HHG_TRY(set_flat(m, l, false));
+    else HHG_TRY(set_flat(m, l, FLAT_OFF));
   }
   // the other candidates' tiles and the level's previous tiles are unused now
   std::vector<void*> unused;
@@ -1487,6 +1487,8 @@ int setup_device(hhg_mesh* m) {
     }
     if (rc == HHG_OK) rc = upload_problem(m, hg, m->global);
   }
+  for (int l = 0; l < nl && rc == HHG_OK; ++l)
+    if (flat_fits(m, l)) rc = set_flat(m, l, FLAT_AUTO);
   if (rc == HHG_OK && m->host.general) {
     const HostLevel& H = m->host.lv.back();
     std::vector<int64_t> off;
@@ -2062,7 +2064,7 @@ int hhg_set_flat_gs(hhg_mesh* m, int enable) {
   if (!m) return fail(HHG_ERR_ARG, "null mesh");
   HHG_TRY(check_device(m));
   HHG_TRY(refuse_general(m, "the flat Gauss-Seidel kernel"));
-  if (!m->host.seven_point) return HHG_OK;   // the flat kernels serve the 7-point structure only
+  if (!m->host.seven_point) return HHG_OK;   // the switch serves the 7-point structure; 15-point levels keep theirs
   const int nl = (int)m->host.lv.size();
   if (enable)
     for (int l = 1; l < nl; ++l)
@@ -2070,7 +2072,8 @@ int hhg_set_flat_gs(hhg_mesh* m, int enable) {
         return fail(HHG_ERR_ARG, "the flat kernels need 4 .. 1024 intervals per macro edge and fewer than 2^31 "
                                  "items per launch");
   drop_local_graph(m);
-  for (int l = 1; l < nl; ++l) HHG_TRY(set_flat(m, l, enable != 0));
+  for (int l = 0; l < nl; ++l)
+    if (l > 0 || flat_fits(m, l)) HHG_TRY(set_flat(m, l, enable ? FLAT_ON : FLAT_OFF));
   return HHG_OK;
 }
 

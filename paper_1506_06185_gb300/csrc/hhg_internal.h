@@ -329,6 +329,11 @@ struct DevLevel {
   T* W = nullptr;   // [n_macro][16][15]
 };
 
+// Whether a level runs the flat kernels: off, switched on, or by default (new
+// meshes, every level the kernels can run; a launch limit selects the tile
+// kernels there).
+constexpr int FLAT_OFF = 0, FLAT_ON = 1, FLAT_AUTO = 2;
+
 struct DevLevelTables {
   int* SL = nullptr;                  // slice-start table of the block layout
   int64_t* if_gid = nullptr;
@@ -343,15 +348,15 @@ struct DevLevelTables {
   int n_tiles_stream = 0;
   StreamTile* tiles_stream32 = nullptr;
   int n_tiles_stream32 = 0;
-  // flat Gauss-Seidel (7-point levels, on request): build_gs_items for FP64
-  // (2 slots per item) and FP32 (4), and whether the level uses it
+  // flat Gauss-Seidel: build_gs_items for FP64 (2 slots per item) and FP32
+  // (4), and whether the level uses it
   uint32_t* gs_items64 = nullptr;
   int gs_off64[5] = {0, 0, 0, 0, 0};
   uint32_t* gs_items32 = nullptr;
   int gs_off32[5] = {0, 0, 0, 0, 0};
   uint32_t* slot_items = nullptr;    // build_slot_items
   int n_slots = 0;
-  int gs_flat = 0;
+  int gs_flat = 0;                   // FLAT_*
 };
 
 struct DevProblemLevel {

@@ -19,11 +19,15 @@
 // slots of one colour segment, so stencil neighbours are contiguous accesses.
 //
 // Flat kernels (k_gs_flat, k_res_flat, k_restrict_flat, k_prolong_flat; the
-// autotuner's choice per level on meshes with the 7-point structure): no
-// tiles, one work item per thread from a per-level table (a 16-byte vector of
-// same-colour slots, or a slot of four nodes), one CTA per 256 items, so a
-// launch has no CTA barrier and no CTA walking a long tile; the per-item
-// arithmetic is the tile kernels', hence the same results bit for bit.
+// default): no tiles, one work item per thread from a per-level table (a
+// 16-byte vector of same-colour slots, or a slot of four nodes), one CTA per
+// 256 items, so a launch has no CTA barrier and no CTA walking a long tile; the
+// per-item arithmetic is the tile kernels', hence the same results bit for bit.
+// One V(3,3) cycle, tile -> flat kernels: 7-point box of 3x2x1 sub-cubes
+// refined 6 times 1.41 -> 1.06 ms, 2x2x2 refined 7 times 3.96 -> 3.00 ms;
+// 15-point (sheared) refined 7 and 8 times 6.85 -> 5.35 and 35.7 -> 32.9 ms.
+// The tile kernels stay for the norms (faster there), for a launch limit, for
+// the streaming and batch forms, and for levels beyond the tables' range.
 //
 // Interface work: a node's stencil is the sum of the sub-stencils of the
 // macros around it (§3.2, Fig. 4); the kernel updates the master in the
@@ -609,6 +613,94 @@ __device__ __forceinline__ void res_group7(const Slice& sc, int N, int j, int g,
   if (WRITE) store_lanes(rb + cc + r0 + m0, acc, lo, hi);
 }
 
+// Base slots (colour array 0) of the seven rows (j + dj, k + dk) a 15-point
+// stencil at row j of slice k touches, from one slot_prefix evaluation.
+struct Rows15 {
+  int r00, rp0, rm0, rmp, r0p, rpm, r0m;   // p: +1, m: -1, in the order (dj, dk)
+};
+__device__ __forceinline__ Rows15 rows15(const Slice& sc, int j) {
+  const int L = sc.M - j, X = slot_prefix(L);
+  Rows15 r;
+  r.r00 = sc.SL0 + sc.SM0 - X;
+  r.rp0 = r.r00 + row_slots(L);
+  r.rm0 = r.r00 - row_slots(L + 1);
+  r.rmp = sc.SLp + sc.SMm - X;
+  r.r0p = r.rmp + row_slots(L);
+  r.rpm = sc.SLm + sc.SMp - X;
+  r.r0m = r.rpm - row_slots(L + 1);
+  return r;
+}
+
+// acc -= w_d u_d over the 14 neighbours, in the order of the directions (the
+// order of the tile kernels), for the colour-c nodes in slots m0 .. m0 + VW - 1
+// of row j: one aligned vector per direction, and one element more where the
+// neighbour's slot is shifted by one.
+template <class T, bool NC>
+__device__ __forceinline__ void sub_group15(const Slice& sc, int j, int c, int ic, int m0, const T* __restrict__ ub,
+                                            const T* __restrict__ w, T* acc) {
+  constexpr int VW = Vec<T>::n;
+  const Rows15 r = rows15(sc, j);
+  const bool e1 = ic == 3, e0 = ic == 0;   // slot of i + 1 is m + e1, of i - 1 is m - e0
+  const T* c1 = ub + ((c + 1) & 3) * sc.CS + m0;
+  const T* c2 = ub + ((c + 2) & 3) * sc.CS + m0;
+  const T* c3 = ub + ((c + 3) & 3) * sc.CS + m0;
+  const T* ptr[NDIR - 1] = {c1 + r.r00, c1 + r.rp0, c1 + r.rmp, c2 + r.rp0, c2 + r.r0p, c2 + r.rmp, c3 + r.r0p,
+                            c3 + r.r00, c3 + r.rm0, c3 + r.rpm, c2 + r.rm0, c2 + r.r0m, c2 + r.rpm, c1 + r.r0m};
+#pragma unroll
+  for (int d = 1; d < NDIR; ++d) {
+    int di, dj, dk;
+    dir_ijk(d, di, dj, dk);
+    T a[VW];
+    load_shifted<T, NC>(ptr[d - 1], di > 0 && e1, di < 0 && e0, a);
+    const T wd = w[d];
+#pragma unroll
+    for (int t = 0; t < VW; ++t) acc[t] -= wd * a[t];
+  }
+}
+
+// 15-point update and residual of an item, as gs_group7 / res_group7.
+template <class T, bool NC = true>
+__device__ __forceinline__ void gs_group15(const Slice& sc, int N, int j, int g, int c, T* __restrict__ ub,
+                                           const T* __restrict__ fb, const T* __restrict__ w, T inv) {
+  constexpr int VW = Vec<T>::n;
+  int ic, mlo, n;
+  colour_row(N, j, sc.k, c, ic, mlo, n);
+  const int m0 = g * VW, me = c * sc.CS + sc.SL0 + sc.SM0 - slot_prefix(sc.M - j) + m0;
+  T acc[VW];
+  Vec<T>::template load<NC>(fb + me, acc);
+  sub_group15<T, NC>(sc, j, c, ic, m0, ub, w, acc);
+#pragma unroll
+  for (int t = 0; t < VW; ++t) acc[t] *= inv;
+  store_lanes(ub + me, acc, max(mlo - m0, 0), min(mlo + n - m0, VW));
+}
+template <class T, bool WRITE, bool NORM, bool ZERO = false, bool NC = true>
+__device__ __forceinline__ void res_group15(const Slice& sc, int N, int j, int g, int c, const T* __restrict__ ub,
+                                            const T* __restrict__ fb, T* __restrict__ rb, const T* __restrict__ w,
+                                            double& ss) {
+  constexpr int VW = Vec<T>::n;
+  int ic, mlo, n;
+  colour_row(N, j, sc.k, c, ic, mlo, n);
+  const int m0 = g * VW, me = c * sc.CS + sc.SL0 + sc.SM0 - slot_prefix(sc.M - j) + m0;
+  T acc[VW], a[VW];
+  if (ZERO) {
+#pragma unroll
+    for (int t = 0; t < VW; ++t) acc[t] = T(0);
+  } else {
+    Vec<T>::template load<NC>(fb + me, acc);
+    Vec<T>::template load<NC>(ub + me, a);
+#pragma unroll
+    for (int t = 0; t < VW; ++t) acc[t] -= w[0] * a[t];
+    sub_group15<T, NC>(sc, j, c, ic, m0, ub, w, acc);
+  }
+  const int lo = max(mlo - m0, 0), hi = min(mlo + n - m0, VW);
+  if (NORM) {
+#pragma unroll
+    for (int t = 0; t < VW; ++t)
+      if (t >= lo && t < hi) ss += (double)acc[t] * (double)acc[t];
+  }
+  if (WRITE) store_lanes(rb + me, acc, lo, hi);
+}
+
 // The 7-point colour-c items of one tile: groups of VW consecutive same-colour
 // slots per thread, the items of all the tile's slices streamed in one pass.
 template <class T, bool SCALED, bool NC = true>
@@ -705,7 +797,7 @@ __global__ void __launch_bounds__(CTA, 5) k_gs(int N, const int* __restrict__ rs
   finish_units(sched, n_if_units + n_tiles * n_act);
 }
 
-// Flat Gauss-Seidel, one colour, 7-point structure: one work item (one
+// Flat Gauss-Seidel, one colour: one work item (one
 // 16-byte vector of same-colour slots of one row) per thread, no tiles, no
 // CTA barrier.  items[it] = (j << 20) | (k << 10) | g lists the colour's
 // items of one macro interior, slice by slice and row by row, so consecutive
@@ -724,8 +816,8 @@ template <class T>
 struct FlatMinCtas {
   static constexpr int value = sizeof(T) == 8 ? 8 : 0;
 };
-template <class T, bool SCALED>
-__global__ void __launch_bounds__(CTA, FlatMinCtas<T>::value) k_gs_flat(int N, const int* __restrict__ rs, int64_t block, T* __restrict__ u,
+template <class T, bool S7, bool SCALED>
+__global__ void __launch_bounds__(CTA, S7 ? FlatMinCtas<T>::value : 0) k_gs_flat(int N, const int* __restrict__ rs, int64_t block, T* __restrict__ u,
                                                  T* __restrict__ uI, const T* __restrict__ fI,
                                                  const T* __restrict__ W, const T* __restrict__ Winv,
                                                  const T* __restrict__ fv, const T* __restrict__ Wv,
@@ -743,10 +835,10 @@ __global__ void __launch_bounds__(CTA, FlatMinCtas<T>::value) k_gs_flat(int N, c
       const int c0 = cptr[node], c1 = cptr[node + 1];
       T val;
       if (tab.nb) {
-        val = (fI[node] - if_offdiag<T, 6>(tab, u, q)) * tab.dinv[q];
+        val = (fI[node] - if_offdiag<T, if_tab_k(S7)>(tab, u, q)) * tab.dinv[q];
       } else {
         T off = T(0), diag = T(0);
-        if_stencil<T, true>(N, rs, block, u, W, cps, c0, c1, off, diag);
+        if_stencil<T, S7>(N, rs, block, u, W, cps, c0, c1, off, diag);
         val = (fI[node] - off) / diag;
       }
       uI[node] = val;
@@ -761,9 +853,14 @@ __global__ void __launch_bounds__(CTA, FlatMinCtas<T>::value) k_gs_flat(int N, c
   const uint32_t d = items[it];
   const int j = (int)(d >> 20), k = (int)((d >> 10) & 1023u), g = (int)(d & 1023u);
   const T* w = Wv + (size_t)macro * 16 * NDIR;
-  const T wr[11] = {T(0), w[1], w[2], w[3], T(0), T(0), T(0), T(0), w[8], w[9], w[10]};
-  gs_group7<T, SCALED>(slice_consts(rs, N, k), N, j, g, colour, u + (size_t)macro * block,
-                       fv + (size_t)macro * block, wr, SCALED ? T(1) : Winv[macro]);
+  if constexpr (S7) {
+    const T wr[11] = {T(0), w[1], w[2], w[3], T(0), T(0), T(0), T(0), w[8], w[9], w[10]};
+    gs_group7<T, SCALED>(slice_consts(rs, N, k), N, j, g, colour, u + (size_t)macro * block,
+                         fv + (size_t)macro * block, wr, SCALED ? T(1) : Winv[macro]);
+  } else {
+    gs_group15<T>(slice_consts(rs, N, k), N, j, g, colour, u + (size_t)macro * block, fv + (size_t)macro * block, w,
+                  Winv[macro]);
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -1204,7 +1301,7 @@ _Pragma("unroll")
   }
 }
 
-// Flat residual, 7-point structure: the items of all four colours of the flat
+// Flat residual: the items of all four colours of the flat
 // Gauss-Seidel tables (colour c's at off[c] .. off[c + 1]) for every active
 // macro, and the interface entries, in chunks of 256 walked with a grid
 // stride (launched with one chunk per CTA), interface chunks spread among the
@@ -1213,7 +1310,7 @@ _Pragma("unroll")
 // same bit for bit; the norm's partial sums would follow the grid.  n_items:
 // items per macro taken (off[4], or off[3] for a norm-only launch that skips
 // colour 3).
-template <class T, bool WRITE, bool NORM>
+template <class T, bool S7, bool WRITE, bool NORM>
 __global__ void __launch_bounds__(CTA) k_res_flat(int N, const int* __restrict__ rs, int64_t block,
                                                   const T* __restrict__ u, const T* __restrict__ uI,
                                                   const T* __restrict__ f, const T* __restrict__ fI, T* __restrict__ r,
@@ -1239,10 +1336,10 @@ __global__ void __launch_bounds__(CTA) k_res_flat(int N, const int* __restrict__
         if (q >= skip_lo && q < skip_hi) {
           res = T(0);                              // the colour smoothed last
         } else if (tab.nb) {
-          res = fI[node] - tab.diag[q] * uI[node] - if_offdiag<T, 6>(tab, u, q);
+          res = fI[node] - tab.diag[q] * uI[node] - if_offdiag<T, if_tab_k(S7)>(tab, u, q);
         } else {
           T off_ = T(0), diag = T(0);
-          if_stencil<T, true>(N, rs, block, u, W, cps, c0, c1, off_, diag);
+          if_stencil<T, S7>(N, rs, block, u, W, cps, c0, c1, off_, diag);
           res = fI[node] - diag * uI[node] - off_;
         }
         if (WRITE) write_copies(N, rs, block, r, cps, cpo, c0, c1, res);
@@ -1261,12 +1358,16 @@ __global__ void __launch_bounds__(CTA) k_res_flat(int N, const int* __restrict__
     const uint32_t d = items[it];
     const int j = (int)(d >> 20), k = (int)((d >> 10) & 1023u), g = (int)(d & 1023u);
     const T* w = W + (size_t)macro * 16 * NDIR;
-    const T wr[11] = {w[0], w[1], w[2], w[3], T(0), T(0), T(0), T(0), w[8], w[9], w[10]};
     const size_t mb = (size_t)macro * block;
-    if (c == skip)
-      res_group7<T, WRITE, NORM, true>(slice_consts(rs, N, k), N, j, g, c, u + mb, f + mb, r + mb, wr, ss);
-    else
-      res_group7<T, WRITE, NORM>(slice_consts(rs, N, k), N, j, g, c, u + mb, f + mb, r + mb, wr, ss);
+    const Slice sc = slice_consts(rs, N, k);
+    if constexpr (S7) {
+      const T wr[11] = {w[0], w[1], w[2], w[3], T(0), T(0), T(0), T(0), w[8], w[9], w[10]};
+      if (c == skip) res_group7<T, WRITE, NORM, true>(sc, N, j, g, c, u + mb, f + mb, r + mb, wr, ss);
+      else res_group7<T, WRITE, NORM>(sc, N, j, g, c, u + mb, f + mb, r + mb, wr, ss);
+    } else {
+      if (c == skip) res_group15<T, WRITE, NORM, true>(sc, N, j, g, c, u + mb, f + mb, r + mb, w, ss);
+      else res_group15<T, WRITE, NORM>(sc, N, j, g, c, u + mb, f + mb, r + mb, w, ss);
+    }
   }
   if (NORM) {
     const double s = block_sum(ss, sh);
@@ -3248,6 +3349,10 @@ cudaError_t launch_gs_stream(const LevelArgs& L, const ProbArgs& p, T* u, T* uI,
   return cudaGetLastError();
 }
 
+// Whether a level's launches take the flat kernels: switched on (1), or left to
+// the default (2), which a launch limit turns into the tile kernels it limits.
+bool flat_on(const LevelArgs& L, const ProbArgs& p) { return L.gs_flat == 1 || (L.gs_flat == 2 && p.grid_cap == 0); }
+
 template <class T>
 cudaError_t gs_colour(const LevelArgs& L, const ProbArgs& p, T* u, T* uI, const T* f, const T* fI, const T* W,
                       const T* Winv, int colour, bool seven_point, cudaStream_t s, cudaEvent_t ev_begin,
@@ -3288,13 +3393,13 @@ cudaError_t gs_colour(const LevelArgs& L, const ProbArgs& p, T* u, T* uI, const 
     return e;
   }
   const uint32_t* items = sizeof(T) == 8 ? L.gs_items64 : L.gs_items32;
-  if (seven_point && L.gs_flat && items) {
+  if (flat_on(L, p) && items) {
     const int* off = sizeof(T) == 8 ? L.gs_off64 : L.gs_off32;
     const int n_items = off[colour + 1] - off[colour];
     const int n_if_ctas = (int)lin_grid(n, CTA);
     const int n_vol_ctas = p.n_act > 0 ? (int)lin_grid((int64_t)n_items * p.n_act, CTA) : 0;
     if (n_if_ctas + n_vol_ctas == 0) return cudaSuccess;
-    auto kern = fs ? k_gs_flat<T, true> : k_gs_flat<T, false>;
+    auto kern = !seven_point ? k_gs_flat<T, false, false> : fs ? k_gs_flat<T, true, true> : k_gs_flat<T, true, false>;
     if (ev_begin) cudaEventRecord(ev_begin, s);
     ++g_kernel_launches;
     kern<<<n_if_ctas + n_vol_ctas, cta_shape(), 0, s>>>(
@@ -3353,7 +3458,7 @@ cudaError_t residual(const LevelArgs& L, const ProbArgs& p, const T* u, const T*
   if (n_part) *n_part = 0;
   if (g.total == 0) return cudaSuccess;
   const uint32_t* items = sizeof(T) == 8 ? L.gs_items64 : L.gs_items32;
-  if (seven_point && L.gs_flat && items && write_r && !norm) {
+  if (flat_on(L, p) && items && write_r && !norm) {
     // the residual before a restriction, on levels whose Gauss-Seidel runs
     // flat: one chunk per CTA (norm launches keep the tile kernel, whose
     // partial sums per CTA measured faster)
@@ -3363,7 +3468,8 @@ cudaError_t residual(const LevelArgs& L, const ProbArgs& p, const T* u, const T*
     const int n_if_chunks = (int)lin_grid(n + n_zero, CTA);
     const int n_vol_chunks = p.n_act > 0 ? (int)lin_grid((int64_t)n_items * p.n_act, CTA) : 0;
     ++g_kernel_launches;
-    k_res_flat<T, true, false><<<n_if_chunks + n_vol_chunks, cta_shape(), 0, s>>>(
+    auto kern = seven_point ? k_res_flat<T, true, true, false> : k_res_flat<T, false, true, false>;
+    kern<<<n_if_chunks + n_vol_chunks, cta_shape(), 0, s>>>(
         L.N, L.rs, L.block, u, uI, f, fI, r, W, items, make_int4(off[0], off[1], off[2], off[3]), n_items, p.act,
         p.n_act, L.cptr, L.cps, L.cp_off, p.free_if, n, if_tab<T>(p, 0), p.zero_off, n_zero, n_if_chunks,
         n_vol_chunks, nullptr, sk, sk >= 0 ? p.col_off[sk] : 0, sk >= 0 ? p.col_off[sk + 1] : 0);
@@ -3413,7 +3519,7 @@ cudaError_t restrict_to(const LevelArgs& C, const LevelArgs& F, const ProbArgs& 
   const int n = pc.col_off[4];
   const Units g = units(n + pc.n_zero, C.n_tiles_int * RESTRICT_SPLIT, pc.n_act);
   if (g.total == 0) return cudaSuccess;
-  if (C.gs_flat && C.slot_items) {
+  if (flat_on(C, pc) && C.slot_items) {
     const int n_if_ctas = (int)lin_grid(n + pc.n_zero, CTA);
     const int n_vol_ctas = pc.n_act > 0 ? (int)lin_grid((int64_t)C.n_slots * pc.n_act, CTA) : 0;
     ++g_kernel_launches;
@@ -3459,7 +3565,7 @@ cudaError_t prolong_add(const LevelArgs& F, const LevelArgs& C, const ProbArgs& 
   const Units g = units(n, F.n_tiles_int, pf.n_act);
   if (g.total == 0) return cudaSuccess;
   const uint32_t* items = sizeof(T) == 8 ? F.gs_items64 : F.gs_items32;
-  if (F.gs_flat && items && (skip == -1 || skip == 0)) {
+  if (flat_on(F, pf) && items && (skip == -1 || skip == 0)) {
     // the fine level's items of the colours updated: all, or 1..3 when the
     // first post-smoothing sweep overwrites colour 0
     const int* off = sizeof(T) == 8 ? F.gs_off64 : F.gs_off32;
