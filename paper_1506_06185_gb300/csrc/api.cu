@@ -325,6 +325,8 @@ ProbArgs pargs(const DevProblem& p, int l) {
   a.td32 = q.td32;
   a.ti32 = q.ti32;
   a.tn = q.tn;
+  a.tptr = q.tptr;
+  a.tlen = q.tlen;
   a.stream_gs = p.stream_gs;
   a.err = p.err;
   a.wait_limit = p.wait_limit;
@@ -334,24 +336,31 @@ ProbArgs pargs(const DevProblem& p, int l) {
 // Interface stencil tables (weights, diagonal, inverse diagonal) of problem
 // level l from the current stencils; allocates on the first call (device
 // pointers null), else overwrites the weights in place (new coefficients).
-// Levels of general meshes, the coarsest level and meshes whose offsets need
-// more than 32 bits keep the per-copy path (tables null).
+// The coarsest level and meshes whose offsets need more than 32 bits keep the
+// per-copy path (tables null).
 int upload_if_tables(hhg_mesh* m, DevProblemLevel& q, int l, int kind, const std::vector<int>& free_if,
-                     const std::vector<int>& pcptr, const std::vector<Copy>& pcopies) {
+                     const std::vector<int>& pcptr, const std::vector<Copy>& pcopies,
+                     const std::vector<int>& class_off = std::vector<int>()) {
   if (l == 0 || free_if.empty()) return HHG_OK;
   const HostLevel& H = m->host.lv[l];
   const std::vector<int>& cptr = kind == 3 ? pcptr : H.if_cptr;
   const std::vector<Copy>& copies = kind == 3 ? pcopies : H.if_copy;
   const int K = m->host.seven_point ? 6 : 14;
-  std::vector<uint32_t> nb;
+  std::vector<uint32_t> nb, ptr;
+  std::vector<int> len;
   std::vector<double> w, dg;
-  if (!build_if_tables(m->host, l, free_if, cptr, copies, K, nb, w, dg)) return HHG_OK;
+  const bool built = m->host.general
+                         ? build_general_if_tables(m->host, l, free_if, class_off, cptr, copies, ptr, len, nb, w, dg)
+                         : build_if_tables(m->host, l, free_if, cptr, copies, K, nb, w, dg);
+  if (!built) return HHG_OK;
   const size_t n = free_if.size();
   std::vector<double> di(n);
   for (size_t i = 0; i < n; ++i) di[i] = 1.0 / dg[i];
   const bool fresh = q.tnb == nullptr;
   if (fresh) {
     HHG_TRY(upload(m, &q.tnb, nb));
+    HHG_TRY(upload(m, &q.tptr, ptr));
+    HHG_TRY(upload(m, &q.tlen, len));
     HHG_TRY(dalloc(m, &q.tw64, w.size()));
     HHG_TRY(dalloc(m, &q.td64, n));
     HHG_TRY(dalloc(m, &q.ti64, n));
@@ -422,7 +431,8 @@ int upload_problem(hhg_mesh* m, const HostProblem& h, DevProblem& d) {
       std::vector<uint32_t> off;
       if (copy_offsets(m->host, (int)l, h.lv[l].copies, off)) HHG_TRY(upload(m, &d.lv[l].cp_off, off));
     }
-    HHG_TRY(upload_if_tables(m, d.lv[l], (int)l, h.kind, h.lv[l].free_if, h.lv[l].cptr, h.lv[l].copies));
+    HHG_TRY(upload_if_tables(m, d.lv[l], (int)l, h.kind, h.lv[l].free_if, h.lv[l].cptr, h.lv[l].copies,
+                             h.lv[l].class_off));
     HHG_TRY(upload(m, &d.lv[l].gptr, h.lv[l].gptr));
     HHG_TRY(upload(m, &d.lv[l].goff, h.lv[l].goff));
     d.lv[l].class_off = h.lv[l].class_off;

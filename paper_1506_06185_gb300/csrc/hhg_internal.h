@@ -313,6 +313,17 @@ bool build_if_tables(const HostMesh& m, int l, const std::vector<int>& free_if, 
                      const std::vector<Copy>& copies, int K, std::vector<uint32_t>& nb, std::vector<double>& w,
                      std::vector<double>& diag);
 
+// The same for a general mesh, whose nodes have any number of neighbours (a
+// face node 14, an edge node some 20, a vertex 50 and more): free_if is taken
+// class by class (class_off), 32 nodes at a time; entry e of node q stands at
+// ptr[q] + 32 e, len[q] entries, the longest of its 32 nodes rounded up to a
+// multiple of four and padded with weight 0.  Returns false (tables empty) when
+// an offset or a position needs more than 32 bits.
+bool build_general_if_tables(const HostMesh& m, int l, const std::vector<int>& free_if,
+                             const std::vector<int>& class_off, const std::vector<int>& cptr,
+                             const std::vector<Copy>& copies, std::vector<uint32_t>& ptr, std::vector<int>& len,
+                             std::vector<uint32_t>& nb, std::vector<double>& w, std::vector<double>& diag);
+
 // ---------------------------------------------------------------------------
 // Device-side structures.
 // ---------------------------------------------------------------------------
@@ -372,7 +383,7 @@ struct DevProblemLevel {
   Copy* cps = nullptr;
   uint32_t* cp_off = nullptr;         // block offsets of those copies (kind 3)
   // interface stencil tables of the free interface nodes (build_if_tables;
-  // null for general meshes and on level 0): tK entries per node,
+  // null on level 0; general meshes: entries at tptr, tlen): tK entries per node,
   // direction-major with stride tn = free_if size; weights, diagonal and its
   // inverse in both precisions (FP32 only on precision-32 meshes)
   uint32_t* tnb = nullptr;
@@ -383,6 +394,8 @@ struct DevProblemLevel {
   float* td32 = nullptr;
   float* ti32 = nullptr;
   int tn = 0;
+  uint32_t* tptr = nullptr;           // general meshes (build_general_if_tables)
+  int* tlen = nullptr;
 };
 
 struct DevProblem {

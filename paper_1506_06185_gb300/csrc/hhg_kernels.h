@@ -56,6 +56,8 @@ struct ProbArgs {
   const float* td32;
   const float* ti32;
   int tn;
+  const uint32_t* tptr;   // general connectivity: start and length of every node's entries
+  const int* tlen;
   int stream_gs;   // 1: 7-point Gauss-Seidel uses the streaming kernel where the level has units
   int* err;        // device flag: set to 1 when a bounded wait of a kernel runs out
   int wait_limit;  // tries of such a wait (about 64 ns apart)

@@ -413,6 +413,10 @@ struct IfTab {
   const T* diag;
   const T* dinv;
   int n;
+  // general connectivity (build_general_if_tables): entry e of list entry q at
+  // ptr[q] + 32 e, len[q] entries (a multiple of four)
+  const uint32_t* ptr;
+  const int* len;
 };
 constexpr int if_tab_k(bool s7) { return s7 ? 6 : 14; }
 
@@ -420,6 +424,16 @@ constexpr int if_tab_k(bool s7) { return s7 ? 6 : 14; }
 template <class T, int K>
 __device__ __forceinline__ T if_offdiag(const IfTab<T>& t, const T* __restrict__ u, int q) {
   T s = T(0);
+  if (K == 14 && t.ptr) {
+    const int n = t.len[q];
+    const uint32_t* nb = t.nb + t.ptr[q];
+    const T* w = t.w + t.ptr[q];
+    for (int e = 0; e < n; e += 4) {
+#pragma unroll
+      for (int x = 0; x < 4; ++x) s += w[32 * (e + x)] * u[nb[32 * (e + x)]];
+    }
+    return s;
+  }
 #pragma unroll
   for (int e = 0; e < K; ++e) s += t.w[(size_t)e * t.n + q] * u[t.nb[(size_t)e * t.n + q]];
   return s;
@@ -2586,14 +2600,16 @@ template <class T>
 IfTab<T> if_tab(const ProbArgs& p, int off);
 template <>
 IfTab<double> if_tab<double>(const ProbArgs& p, int off) {
-  IfTab<double> t{nullptr, nullptr, nullptr, nullptr, 0};
-  if (p.tnb && p.tw64) t = IfTab<double>{p.tnb + off, p.tw64 + off, p.td64 + off, p.ti64 + off, p.tn};
+  IfTab<double> t{nullptr, nullptr, nullptr, nullptr, 0, nullptr, nullptr};
+  if (p.tnb && p.tw64) t = IfTab<double>{p.tnb + (p.tptr ? 0 : off), p.tw64 + (p.tptr ? 0 : off), p.td64 + off, p.ti64 + off, p.tn,
+                                          p.tptr ? p.tptr + off : nullptr, p.tlen ? p.tlen + off : nullptr};
   return t;
 }
 template <>
 IfTab<float> if_tab<float>(const ProbArgs& p, int off) {
-  IfTab<float> t{nullptr, nullptr, nullptr, nullptr, 0};
-  if (p.tnb && p.tw32) t = IfTab<float>{p.tnb + off, p.tw32 + off, p.td32 + off, p.ti32 + off, p.tn};
+  IfTab<float> t{nullptr, nullptr, nullptr, nullptr, 0, nullptr, nullptr};
+  if (p.tnb && p.tw32) t = IfTab<float>{p.tnb + (p.tptr ? 0 : off), p.tw32 + (p.tptr ? 0 : off), p.td32 + off, p.ti32 + off, p.tn,
+                                          p.tptr ? p.tptr + off : nullptr, p.tlen ? p.tlen + off : nullptr};
   return t;
 }
 inline dim3 cta_shape() { return dim3(TILE_SLOTS, TILE_ROWS); }
@@ -2661,14 +2677,16 @@ template <class T>
 __device__ __forceinline__ IfTab<T> dev_if_tab(const ProbArgs& p, int off);
 template <>
 __device__ __forceinline__ IfTab<double> dev_if_tab<double>(const ProbArgs& p, int off) {
-  IfTab<double> t{nullptr, nullptr, nullptr, nullptr, 0};
-  if (p.tnb && p.tw64) t = IfTab<double>{p.tnb + off, p.tw64 + off, p.td64 + off, p.ti64 + off, p.tn};
+  IfTab<double> t{nullptr, nullptr, nullptr, nullptr, 0, nullptr, nullptr};
+  if (p.tnb && p.tw64) t = IfTab<double>{p.tnb + (p.tptr ? 0 : off), p.tw64 + (p.tptr ? 0 : off), p.td64 + off, p.ti64 + off, p.tn,
+                                          p.tptr ? p.tptr + off : nullptr, p.tlen ? p.tlen + off : nullptr};
   return t;
 }
 template <>
 __device__ __forceinline__ IfTab<float> dev_if_tab<float>(const ProbArgs& p, int off) {
-  IfTab<float> t{nullptr, nullptr, nullptr, nullptr, 0};
-  if (p.tnb && p.tw32) t = IfTab<float>{p.tnb + off, p.tw32 + off, p.td32 + off, p.ti32 + off, p.tn};
+  IfTab<float> t{nullptr, nullptr, nullptr, nullptr, 0, nullptr, nullptr};
+  if (p.tnb && p.tw32) t = IfTab<float>{p.tnb + (p.tptr ? 0 : off), p.tw32 + (p.tptr ? 0 : off), p.td32 + off, p.ti32 + off, p.tn,
+                                          p.tptr ? p.tptr + off : nullptr, p.tlen ? p.tlen + off : nullptr};
   return t;
 }
 

@@ -725,6 +725,81 @@ bool build_if_tables(const HostMesh& m, int l, const std::vector<int>& free_if, 
   return true;
 }
 
+bool build_general_if_tables(const HostMesh& m, int l, const std::vector<int>& free_if,
+                             const std::vector<int>& class_off, const std::vector<int>& cptr,
+                             const std::vector<Copy>& copies, std::vector<uint32_t>& ptr, std::vector<int>& len,
+                             std::vector<uint32_t>& nb, std::vector<double>& w, std::vector<double>& diag) {
+  const HostLevel& L = m.lv[l];
+  const int N = L.N;
+  const size_t n = free_if.size();
+  ptr.clear();
+  len.clear();
+  nb.clear();
+  w.clear();
+  diag.clear();
+  if ((uint64_t)m.n_macro * (uint64_t)L.block > 0x7fffffffull) return false;
+  auto offset = [&](int t, int i, int j, int k) {
+    return (uint32_t)((int64_t)t * L.block + lidx(L.SL.data(), N, i, j, k));
+  };
+  // interface node at every block offset (-1: a volume node)
+  std::vector<int> node_at((size_t)m.n_macro * L.block, -1);
+  for (int q = 0; q < L.n_if; ++q)
+    for (int c = L.if_cptr[q]; c < L.if_cptr[q + 1]; ++c) {
+      const Copy& cp = L.if_copy[c];
+      node_at[offset(cp.macro, cp.i, cp.j, cp.k)] = q;
+    }
+  struct Ent {
+    int64_t id;   // node, or n_if + offset of a volume node
+    double w;
+    uint32_t off;
+  };
+  std::vector<std::vector<Ent>> ent(32);
+  ptr.resize(n);
+  len.resize(n);
+  diag.assign(n, 0.0);
+  for (size_t c = 0; c + 1 < class_off.size(); ++c)
+    for (int q0 = class_off[c]; q0 < class_off[c + 1]; q0 += 32) {
+      const int q1 = std::min(q0 + 32, class_off[c + 1]);
+      size_t longest = 0;
+      for (int q = q0; q < q1; ++q) {
+        std::vector<Ent>& E = ent[q - q0];
+        E.clear();
+        for (int x = cptr[free_if[q]]; x < cptr[free_if[q] + 1]; ++x) {
+          const Copy& cp = copies[x];
+          const double* wm = &L.W[((size_t)cp.macro * 16 + node_class(cp.i, cp.j, cp.k, N)) * NDIR];
+          diag[q] += wm[0];
+          for (int d = 1; d < NDIR; ++d) {
+            int di, dj, dk;
+            dir_ijk(d, di, dj, dk);
+            if (wm[d] == 0.0 || !in_lattice(cp.i + di, cp.j + dj, cp.k + dk, N)) continue;
+            const uint32_t off = offset(cp.macro, cp.i + di, cp.j + dj, cp.k + dk);
+            const int64_t id = node_at[off] >= 0 ? node_at[off] : (int64_t)L.n_if + off;
+            auto it = std::find_if(E.begin(), E.end(), [&](const Ent& e) { return e.id == id; });
+            if (it != E.end()) it->w += wm[d];
+            else E.push_back(Ent{id, wm[d], off});
+          }
+        }
+        longest = std::max(longest, E.size());
+      }
+      longest = (longest + 3) & ~size_t(3);
+      const size_t base = nb.size();
+      if (base + 32 * longest > 0x7fffffffull) return false;
+      nb.resize(base + 32 * longest, 0);
+      w.resize(base + 32 * longest, 0.0);
+      for (int q = q0; q < q1; ++q) {
+        const std::vector<Ent>& E = ent[q - q0];
+        const Copy& own = copies[cptr[free_if[q]]];
+        ptr[q] = (uint32_t)(base + (q - q0));
+        len[q] = (int)longest;
+        for (size_t e = 0; e < longest; ++e) {
+          nb[ptr[q] + 32 * e] = e < E.size() ? E[e].off : offset(own.macro, own.i, own.j, own.k);
+          w[ptr[q] + 32 * e] = e < E.size() ? E[e].w : 0.0;
+        }
+      }
+    }
+  return true;
+}
+
 void build_problem(const HostMesh& m, int kind, const std::vector<unsigned char>& faulty, HostProblem& p) {
   p = HostProblem();
   p.kind = kind;
