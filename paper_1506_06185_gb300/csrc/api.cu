@@ -123,6 +123,7 @@ struct hhg_mesh {
   cudaGraphExec_t local_exec = nullptr;
   long long local_kernels = 0;  // kernels in the captured cycle
   bool local_failed = false;
+  int local_overlap = 1;
   bool local_mixed = false;
   int local_pre = 0, local_post = 0, local_maxit = 0;
   double local_rtol = 0.0;
@@ -327,6 +328,7 @@ ProbArgs pargs(const DevProblem& p, int l) {
   a.tn = q.tn;
   a.tptr = q.tptr;
   a.tlen = q.tlen;
+  a.overlap = p.overlap;
   a.stream_gs = p.stream_gs;
   a.err = p.err;
   a.wait_limit = p.wait_limit;
@@ -777,6 +779,19 @@ void drop_local_graph(hhg_mesh* m) {
   m->local_failed = false;
 }
 
+// Whether Omega_F's launches may overlap each other beside the cycles of the
+// problem `other` on another stream.  Where both sides' finest sweeps fill the
+// GPU the other side is what the recovery waits for, and a denser Omega_F at the
+// higher priority only slows it down (cube refined 8 times, 12 + 3 cycles: the
+// two sides take 29.7 / 60.8 ms with, 35.6 / 55.4 ms without); elsewhere the
+// latency of Omega_F's launches counts (refined 6 times: 5.6 / 5.6 against 6.3 /
+// 2.2 ms; one macro of 3x3x3 sub-cubes in a DN solve: 16.2 against 18.2 ms).
+int overlap_beside(const hhg_mesh* m, const DevProblem& other) {
+  // CTAs of 256 vectors in one colour of one macro: about N^3 / 48 vectors
+  const int64_t N = m->host.lv.back().N, per_macro = N * N * N / (48 * 256);
+  return std::min(m->faulty.n_act, other.n_act) * per_macro <= 2432 ? 1 : 0;
+}
+
 // n cycles of the faulty problem on stream ls: the first one directly (it
 // also fills the launch-shape caches), the others as replays of one captured
 // cycle (captured on the mesh's own stream, so ls may be the legacy stream).
@@ -785,7 +800,7 @@ int local_cycles(hhg_mesh* m, int n, bool mixed, int pre, int post, double cg_rt
   if (n <= 0) return HHG_OK;
   HHG_TRY(cycle(m, m->faulty, mixed, pre, post, cg_rtol, cg_maxit, ls));
   if (n == 1) return HHG_OK;
-  const bool same = m->local_mixed == mixed && m->local_pre == pre && m->local_post == post &&
+  const bool same = m->local_overlap == m->faulty.overlap && m->local_mixed == mixed && m->local_pre == pre && m->local_post == post &&
                     m->local_rtol == cg_rtol && m->local_maxit == cg_maxit;
   if (!same) drop_local_graph(m);
   // inside a caller's own stream capture the cycles are recorded directly
@@ -814,6 +829,7 @@ int local_cycles(hhg_mesh* m, int n, bool mixed, int pre, int post, double cg_rt
       m->local_failed = true;
     }
     m->local_mixed = mixed;
+    m->local_overlap = m->faulty.overlap;
     m->local_pre = pre;
     m->local_post = post;
     m->local_rtol = cg_rtol;
@@ -973,6 +989,7 @@ int recover(hhg_mesh* m, int n_local, int n_global, bool mixed, int pre, int pos
     HHG_CUDA(cudaEventRecord(m->ev_fork, s));
     HHG_CUDA(cudaStreamWaitEvent(ls, m->ev_fork, 0));
   }
+  m->faulty.overlap = n_global > 0 ? overlap_beside(m, m->healthy) : 1;
   if (timed) HHG_CUDA(cudaEventRecord(a0, ls));
   HHG_TRY(local_cycles(m, n_local, mixed, pre, post, cg_rtol, cg_maxit, ls));
   if (timed) HHG_CUDA(cudaEventRecord(a1, ls));
@@ -1072,6 +1089,7 @@ int recover_dn(hhg_mesh* m, int n_global, double eta, bool mixed, int pre, int p
                           m->dn.fI_top, s));
   HHG_CUDA(cudaEventRecord(m->ev_dn_e, s));
   if (timed) HHG_CUDA(cudaEventRecord(b0, s));
+  m->faulty.overlap = overlap_beside(m, m->dn);
   int total = 0;
   for (int j = 1; j <= n_global; ++j) {
     const int cyc = (int)std::ceil(j * eta) - (int)std::ceil((j - 1) * eta);
@@ -1305,6 +1323,7 @@ int tune_level(hhg_mesh* m, int l, int reps, cudaStream_t s, int* best_out) {
 }
 
 int capture_task(hhg_mesh* m, int cycles, bool recovery, bool mixed, cudaStream_t s) {
+  m->faulty.overlap = 1;
   if (recovery) {
     HHG_TRY(inject(m, s));
     for (int c = 0; c < cycles; ++c) HHG_TRY(cycle(m, m->faulty, mixed, 3, 3, 1e-12, 1000, s));

@@ -403,6 +403,7 @@ struct DevProblem {
   int* sched = nullptr;               // counters of the dynamic walks (kernels.cu): next unit,
                                       // finished CTAs, completed dynamic launches
   int grid_cap = 0;                   // CTAs per fused launch at most (0: resident CTAs)
+  int overlap = 1;                    // small launches may overlap their predecessor's end
   int stream_gs = 0;                  // streaming 7-point Gauss-Seidel where a level has units
   int* err = nullptr;                 // the mesh's device error flag (bounded waits)
   int wait_limit = 1 << 24;           // tries of a bounded device wait

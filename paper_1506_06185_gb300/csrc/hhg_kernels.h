@@ -58,6 +58,7 @@ struct ProbArgs {
   int tn;
   const uint32_t* tptr;   // general connectivity: start and length of every node's entries
   const int* tlen;
+  int overlap;     // small launches may overlap their predecessor's end
   int stream_gs;   // 1: 7-point Gauss-Seidel uses the streaming kernel where the level has units
   int* err;        // device flag: set to 1 when a bounded wait of a kernel runs out
   int wait_limit;  // tries of such a wait (about 64 ns apart)

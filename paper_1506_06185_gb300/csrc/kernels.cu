@@ -52,6 +52,16 @@ namespace {
 
 constexpr int CTA = TILE_ROWS * TILE_SLOTS;   // 256 threads, 32 x 8
 
+// Programmatic dependent launch: the kernels of a cycle are launched so that a
+// kernel's CTAs may start while its predecessor in the stream drains
+// (launch_next lets the successor start as early as that).  after_previous
+// returns when the predecessor has completed and its writes are visible; before
+// it a kernel touches only tables written at set-up (work items, active macros,
+// lists, copy pointers, stencil weights), which host-synchronous copies wrote.
+// Every kernel calls it, so completion stays in stream order.
+__device__ __forceinline__ void launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void after_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // 7-point structure: only the three chain axes (and negatives) are non-zero.
 __host__ __device__ constexpr bool used_dir(int d, bool s7) {
   return !s7 || d == 1 || d == 2 || d == 3 || d == 8 || d == 9 || d == 10;
@@ -747,6 +757,8 @@ __global__ void __launch_bounds__(CTA, 5) k_gs(int N, const int* __restrict__ rs
                                             const Copy* __restrict__ cps, const uint32_t* __restrict__ cpo,
                                             const int* __restrict__ list, int n_list, IfTab<T> tab,
                                             int n_if_units, int* __restrict__ sched) {
+  launch_next();
+  after_previous();
   __shared__ int s_pre2[MAX_SLABS][33];
   __shared__ int s_pre_tot[MAX_SLABS + 1];
   __shared__ int s_unit;
@@ -830,7 +842,7 @@ template <class T>
 struct FlatMinCtas {
   static constexpr int value = sizeof(T) == 8 ? 8 : 0;
 };
-template <class T, bool S7, bool SCALED>
+template <class T, bool S7, bool SCALED, bool DEP>
 __global__ void __launch_bounds__(CTA, S7 ? FlatMinCtas<T>::value : 0) k_gs_flat(int N, const int* __restrict__ rs, int64_t block, T* __restrict__ u,
                                                  T* __restrict__ uI, const T* __restrict__ fI,
                                                  const T* __restrict__ W, const T* __restrict__ Winv,
@@ -840,6 +852,7 @@ __global__ void __launch_bounds__(CTA, S7 ? FlatMinCtas<T>::value : 0) k_gs_flat
                                                  const int* __restrict__ cptr, const Copy* __restrict__ cps,
                                                  const uint32_t* __restrict__ cpo, const int* __restrict__ list,
                                                  int n_list, IfTab<T> tab, int n_if_ctas, int n_vol_ctas) {
+  if (DEP) launch_next();
   int vb = 0;
   const int ib = spread_position((int)blockIdx.x, n_if_ctas, n_vol_ctas, vb);
   if (ib >= 0) {
@@ -847,6 +860,7 @@ __global__ void __launch_bounds__(CTA, S7 ? FlatMinCtas<T>::value : 0) k_gs_flat
     if (q < n_list) {
       const int node = list[q];
       const int c0 = cptr[node], c1 = cptr[node + 1];
+      if (DEP) after_previous();
       T val;
       if (tab.nb) {
         val = (fI[node] - if_offdiag<T, if_tab_k(S7)>(tab, u, q)) * tab.dinv[q];
@@ -869,11 +883,19 @@ __global__ void __launch_bounds__(CTA, S7 ? FlatMinCtas<T>::value : 0) k_gs_flat
   const T* w = Wv + (size_t)macro * 16 * NDIR;
   if constexpr (S7) {
     const T wr[11] = {T(0), w[1], w[2], w[3], T(0), T(0), T(0), T(0), w[8], w[9], w[10]};
-    gs_group7<T, SCALED>(slice_consts(rs, N, k), N, j, g, colour, u + (size_t)macro * block,
-                         fv + (size_t)macro * block, wr, SCALED ? T(1) : Winv[macro]);
+    if constexpr (DEP) {
+      const Slice sc = slice_consts(rs, N, k);
+      const T inv = SCALED ? T(1) : Winv[macro];
+      after_previous();
+      gs_group7<T, SCALED>(sc, N, j, g, colour, u + (size_t)macro * block, fv + (size_t)macro * block, wr, inv);
+    } else {
+      gs_group7<T, SCALED>(slice_consts(rs, N, k), N, j, g, colour, u + (size_t)macro * block,
+                           fv + (size_t)macro * block, wr, SCALED ? T(1) : Winv[macro]);
+    }
   } else {
-    gs_group15<T>(slice_consts(rs, N, k), N, j, g, colour, u + (size_t)macro * block, fv + (size_t)macro * block, w,
-                  Winv[macro]);
+    const Slice sc = slice_consts(rs, N, k);
+    if (DEP) after_previous();
+    gs_group15<T>(sc, N, j, g, colour, u + (size_t)macro * block, fv + (size_t)macro * block, w, Winv[macro]);
   }
 }
 
@@ -1044,6 +1066,8 @@ __global__ void __launch_bounds__(STREAM_CTA) k_gs_stream(
     int n_act, int colour, const int* __restrict__ cptr, const Copy* __restrict__ cps,
     const uint32_t* __restrict__ cpo, const int* __restrict__ list, int n_list, IfTab<T> tab, int n_if_units,
     int* __restrict__ sched, int slot, int wait_limit, int* __restrict__ err) {
+  launch_next();
+  after_previous();
   extern __shared__ __align__(128) unsigned char s_dyn[];
   T* const buf = reinterpret_cast<T*>(s_dyn) + STREAM_PAD;
   __shared__ __align__(8) uint64_t full[3], empty[3];
@@ -1232,6 +1256,8 @@ __global__ void __launch_bounds__(CTA, 4) k_res(int N, const int* __restrict__ r
                                              const int64_t* __restrict__ zero_off, int n_zero, int n_if_units,
                                              double* __restrict__ partial, int* __restrict__ sched, int skip,
                                              int skip_lo, int skip_hi) {
+  launch_next();
+  after_previous();
   __shared__ int s_pre2[MAX_SLABS][33];
   __shared__ int s_pre_tot[MAX_SLABS + 1];
   __shared__ double sh[32];
@@ -1324,7 +1350,7 @@ _Pragma("unroll")
 // same bit for bit; the norm's partial sums would follow the grid.  n_items:
 // items per macro taken (off[4], or off[3] for a norm-only launch that skips
 // colour 3).
-template <class T, bool S7, bool WRITE, bool NORM>
+template <class T, bool S7, bool WRITE, bool NORM, bool DEP>
 __global__ void __launch_bounds__(CTA) k_res_flat(int N, const int* __restrict__ rs, int64_t block,
                                                   const T* __restrict__ u, const T* __restrict__ uI,
                                                   const T* __restrict__ f, const T* __restrict__ fI, T* __restrict__ r,
@@ -1338,6 +1364,8 @@ __global__ void __launch_bounds__(CTA) k_res_flat(int N, const int* __restrict__
   __shared__ double sh[32];
   double ss = 0.0;
   const int n_vol = n_items * n_act;
+  if (DEP) launch_next();
+  if (DEP) after_previous();
   for (int chunk = blockIdx.x; chunk < n_if_chunks + n_vol_chunks; chunk += gridDim.x) {
     int vc = 0;
     const int ic = spread_position(chunk, n_if_chunks, n_vol_chunks, vc);
@@ -1479,6 +1507,8 @@ __global__ void __launch_bounds__(CTA, 4) k_restrict(int Nc, const int* __restri
                                                   const int* __restrict__ list, int n_list,
                                                   const int64_t* __restrict__ gather,
                                                   const int64_t* __restrict__ zero_off, int n_zero, int n_if_units, int* __restrict__ sched) {
+  launch_next();
+  after_previous();
   __shared__ int s_pre2[MAX_SLABS][33];
   __shared__ int s_pre_tot[MAX_SLABS + 1];
   __shared__ int s_unit;
@@ -1680,6 +1710,8 @@ __global__ void __launch_bounds__(CTA) k_prolong(int Nf, const int* __restrict__
                                                  const int* __restrict__ list,
                                                  int n_list, int n_if_units, int* __restrict__ sched, int skip,
                                                  int if_lo, int if_hi) {
+  launch_next();
+  after_previous();
   __shared__ int s_pre2[MAX_SLABS][33];
   __shared__ int s_pre_tot[MAX_SLABS + 1];
   __shared__ int s_unit;
@@ -1712,7 +1744,7 @@ __global__ void __launch_bounds__(CTA) k_prolong(int Nf, const int* __restrict__
 // Gauss-Seidel items of the colours it updates (one 16-byte vector of
 // same-colour fine nodes per thread, prolong_group).  Same arithmetic per
 // node as k_restrict / k_prolong, so the same values bit for bit.
-template <class T>
+template <class T, bool DEP>
 __global__ void __launch_bounds__(CTA) k_restrict_flat(int Nc, const int* __restrict__ rsc, int64_t bc,
                                                        T* __restrict__ fc, T* __restrict__ fIc, T* __restrict__ uc,
                                                        T* __restrict__ uIc, int Nf, const int* __restrict__ rsf,
@@ -1724,9 +1756,11 @@ __global__ void __launch_bounds__(CTA) k_restrict_flat(int Nc, const int* __rest
                                                        int n_list, const int64_t* __restrict__ gather,
                                                        const int64_t* __restrict__ zero_off, int n_zero,
                                                        int n_if_ctas, int n_vol_ctas) {
+  if (DEP) launch_next();
   int vb = 0;
   const int ib = spread_position((int)blockIdx.x, n_if_ctas, n_vol_ctas, vb);
   if (ib >= 0) {
+    if (DEP) after_previous();
     const int q = ib * CTA + tid256();
     if (q < n_list) {
       const int node = list[q];
@@ -1749,6 +1783,7 @@ __global__ void __launch_bounds__(CTA) k_restrict_flat(int Nc, const int* __rest
   const int a = v / n_slots, it = v - a * n_slots;
   const int macro = act[a];
   const uint32_t d = slots[it];
+  if (DEP) after_previous();
   restrict_slot<T, true>(Nc, rsc, Nf, rsf, (int)(d >> 20), (int)((d >> 10) & 1023u), (int)(d & 1023u),
                          rf + (size_t)macro * bf, fc + (size_t)macro * bc, uc + (size_t)macro * bc);
 }
@@ -1757,7 +1792,7 @@ __global__ void __launch_bounds__(CTA) k_restrict_flat(int Nc, const int* __rest
 // 3 (colour-major, from off[first_c] on); off holds the starts of the later
 // colours relative to that (n_items where there is none), to find an item's
 // colour.
-template <class T>
+template <class T, bool DEP>
 __global__ void __launch_bounds__(CTA) k_prolong_flat(int Nf, const int* __restrict__ rsf, int64_t bf,
                                                       T* __restrict__ uf, T* __restrict__ uIf, int Nc,
                                                       const int* __restrict__ rsc, int64_t bc,
@@ -1768,9 +1803,11 @@ __global__ void __launch_bounds__(CTA) k_prolong_flat(int Nf, const int* __restr
                                                       const uint32_t* __restrict__ cpo,
                                                       const int* __restrict__ list, int n_list, int if_lo, int if_hi,
                                                       int n_if_ctas, int n_vol_ctas) {
+  if (DEP) launch_next();
   int vb = 0;
   const int ib = spread_position((int)blockIdx.x, n_if_ctas, n_vol_ctas, vb);
   if (ib >= 0) {
+    if (DEP) after_previous();
     const int q = ib * CTA + tid256();
     if (q < n_list && (q < if_lo || q >= if_hi)) {
       const int node = list[q];
@@ -1788,6 +1825,7 @@ __global__ void __launch_bounds__(CTA) k_prolong_flat(int Nf, const int* __restr
   const int c = first_c + (it >= off.x) + (it >= off.y) + (it >= off.z);
   const int macro = act[a];
   const uint32_t d = items[it];
+  if (DEP) after_previous();
   prolong_group<T, true>(Nf, rsf, Nc, rsc, (int)(d >> 20), (int)((d >> 10) & 1023u), (int)(d & 1023u), c,
                          uf + (size_t)macro * bf, uc + (size_t)macro * bc);
 }
@@ -1807,6 +1845,8 @@ __global__ void __launch_bounds__(CTA) k_res_f32(int N, const int* __restrict__ 
                                                  const int* __restrict__ list, int n_list, IfTab<double> tab,
                                                  int n_if_units, double* __restrict__ partial,
                                                  int* __restrict__ sched) {
+  launch_next();
+  after_previous();
   __shared__ int s_pre2[MAX_SLABS][33];
   __shared__ int s_pre_tot[MAX_SLABS + 1];
   __shared__ double sh[32];
@@ -1877,6 +1917,8 @@ _Pragma("unroll")
 // copies stay equal to their masters.  Blocks are multiples of 256 slots.
 __global__ void __launch_bounds__(256) k_add_corr_blocks(double* __restrict__ u, const float* __restrict__ e,
                                                         int64_t block, const int* __restrict__ act) {
+  launch_next();
+  after_previous();
   const size_t base = (size_t)act[blockIdx.y] * block;
   double2* ub = reinterpret_cast<double2*>(u + base);
   const float2* eb = reinterpret_cast<const float2*>(e + base);
@@ -1892,6 +1934,8 @@ __global__ void __launch_bounds__(256) k_add_corr_blocks(double* __restrict__ u,
 // uI[list[q]] += eI[list[q]] for the free interface masters.
 __global__ void k_add_corr_masters(double* __restrict__ uI, const float* __restrict__ eI, const int* __restrict__ list,
                                    int n) {
+  launch_next();
+  after_previous();
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q < n) {
     const int node = list[q];
@@ -2107,6 +2151,8 @@ __global__ void __launch_bounds__(CG_THREADS) k_cg(int n, const int* __restrict_
                                                    T* __restrict__ uI, double* __restrict__ work,
                                                    const double* __restrict__ dinv, double rtol, int maxit,
                                                    int* __restrict__ iters) {
+  launch_next();
+  after_previous();
   __shared__ double red[64];
   cg_one_cta<T>(n, rowptr, col, val, fsrc, f, fI, uptr, udst, umaster, u, uI, work, work + n, work + 2 * (size_t)n,
                 work + 3 * (size_t)n, dinv, rtol, maxit, iters, red);
@@ -2190,6 +2236,7 @@ template <class T, int NB, int KC, bool JAC>
 __global__ void __launch_bounds__(NB > 0 ? CG_THREADS + 32 : 1024) k_cg_cluster(CgArgs A, const T* __restrict__ f,
                                                                 const T* __restrict__ fI, T* __restrict__ u,
                                                                 T* __restrict__ uI) {
+  launch_next();
   extern __shared__ double s_cg[];
   __shared__ double s_alpha, s_beta;
   __shared__ int s_go;
@@ -2316,6 +2363,7 @@ __global__ void __launch_bounds__(NB > 0 ? CG_THREADS + 32 : 1024) k_cg_cluster(
   double* gp = gx + (NB > 0 ? 0 : (size_t)A.n);
   double* gs = gp + (NB > 0 ? 0 : (size_t)A.n);
   double* gw = gs + (NB > 0 ? 0 : (size_t)A.n);
+  after_previous();
   barrier();   // every CTA of the cluster runs before its memory is written
   each_sum(peer0, [&](int i, int g, int q) {
     double v = 0.0;
@@ -2413,6 +2461,8 @@ __global__ void __launch_bounds__(CTA) k_grad(int N, const int* __restrict__ rs,
                                               const double* __restrict__ u, const double* __restrict__ lam,
                                               const double* __restrict__ W, const Tile* __restrict__ tiles,
                                               double* __restrict__ partial) {
+  launch_next();
+  after_previous();
   __shared__ double sh[32];
   const Tile t = tiles[blockIdx.x];
   const int macro = blockIdx.y;
@@ -2447,6 +2497,8 @@ __global__ void __launch_bounds__(CTA) k_grad(int N, const int* __restrict__ rs,
 }
 
 __global__ void k_reduce_per_macro(const double* __restrict__ partial, int n_per, double* __restrict__ out) {
+  launch_next();
+  after_previous();
   __shared__ double sh[33];
   double s = 0.0;
   const double* p = partial + (size_t)blockIdx.x * n_per;
@@ -2456,6 +2508,8 @@ __global__ void k_reduce_per_macro(const double* __restrict__ partial, int n_per
 }
 
 __global__ void k_reduce(const double* __restrict__ partial, int n, double* __restrict__ out) {
+  launch_next();
+  after_previous();
   __shared__ double sh[33];
   double s = 0.0;
   for (int q = threadIdx.x; q < n; q += blockDim.x) s += partial[q];
@@ -2493,6 +2547,8 @@ template <class T>
 __global__ void __launch_bounds__(CTA) k_import_vol(int N, const int* __restrict__ rs, int64_t block, const MacroGeo* __restrict__ geo,
                                                     int64_t nx, int64_t ny, const double* __restrict__ g,
                                                     T* __restrict__ dst, const Tile* __restrict__ tiles, bool closed) {
+  launch_next();
+  after_previous();
   const Tile t = tiles[blockIdx.x];
   const int macro = blockIdx.y;
   const int k = t.k;
@@ -2514,6 +2570,8 @@ template <class T>
 __global__ void __launch_bounds__(CTA) k_export_vol(int N, const int* __restrict__ rs, int64_t block, const MacroGeo* __restrict__ geo,
                                                     int64_t nx, int64_t ny, const T* __restrict__ src,
                                                     double* __restrict__ g, const Tile* __restrict__ tiles) {
+  launch_next();
+  after_previous();
   const Tile t = tiles[blockIdx.x];
   const int macro = blockIdx.y;
   const int k = t.k;
@@ -2532,12 +2590,16 @@ __global__ void __launch_bounds__(CTA) k_export_vol(int N, const int* __restrict
 
 template <class T>
 __global__ void k_import_if(const int64_t* __restrict__ gid, int n, const double* __restrict__ g, T* __restrict__ m) {
+  launch_next();
+  after_previous();
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q < n) m[q] = (T)g[gid[q]];
 }
 
 template <class T>
 __global__ void k_export_if(const int64_t* __restrict__ gid, int n, const T* __restrict__ m, double* __restrict__ g) {
+  launch_next();
+  after_previous();
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q < n) g[gid[q]] = (double)m[q];
 }
@@ -2548,6 +2610,8 @@ template <bool S7>
 __global__ void k_if_apply(int N, const int* __restrict__ rs, int64_t block, const double* __restrict__ u,
                            const double* __restrict__ uI, const double* __restrict__ W, const int* __restrict__ cptr,
                            const Copy* __restrict__ cps, const int* __restrict__ list, int n, double* __restrict__ out) {
+  launch_next();
+  after_previous();
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= n) return;
   const int node = list[q];
@@ -2558,30 +2622,40 @@ __global__ void k_if_apply(int N, const int* __restrict__ rs, int64_t block, con
 
 __global__ void k_copy_listed(const double* __restrict__ src, double* __restrict__ dst, const int* __restrict__ idx,
                               int n) {
+  launch_next();
+  after_previous();
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q < n) dst[idx[q]] = src[idx[q]];
 }
 
 __global__ void k_scale_blocks(const double* __restrict__ f, const double* __restrict__ winv,
                                double* __restrict__ out, int n_macro, int64_t block) {
+  launch_next();
+  after_previous();
   const int64_t total = (int64_t)n_macro * block;
   for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < total; q += (int64_t)gridDim.x * blockDim.x)
     out[q] = f[q] * winv[q / block];
 }
 
 __global__ void k_set_masters_zero(double* __restrict__ uI, const int* __restrict__ ids, int n) {
+  launch_next();
+  after_previous();
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q < n) uI[ids[q]] = 0.0;
 }
 
 __global__ void k_restore(double* __restrict__ u, const double* __restrict__ uI, const int64_t* __restrict__ off,
                           const int* __restrict__ master, int n) {
+  launch_next();
+  after_previous();
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q < n) u[off[q]] = uI[master[q]];
 }
 
 template <class T>
 __global__ void k_zero_blocks(T* __restrict__ u, int64_t block, const int* __restrict__ act) {
+  launch_next();
+  after_previous();
   T* b = u + (size_t)act[blockIdx.y] * block;
   for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < block; q += (int64_t)gridDim.x * blockDim.x)
     b[q] = T(0);
@@ -2589,8 +2663,37 @@ __global__ void k_zero_blocks(T* __restrict__ u, int64_t block, const int* __res
 
 template <class T>
 __global__ void k_zero_list(T* __restrict__ uI, const int* __restrict__ list, int n) {
+  launch_next();
+  after_previous();
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q < n) uI[list[q]] = T(0);
+}
+
+// Launches of at most this many CTAs (or work units) may overlap their
+// predecessor's end (see launch_next): on levels of up to two waves of CTAs the
+// launch latency counts (one cycle of 2x2x2 sub-cubes refined 5 times 0.66 ->
+// 0.46 ms, 7 times 2.98 -> 2.74 ms, 8 times 15.86 -> 15.60 ms).  Larger ones run
+// without: they gain under 1%, their waiting CTAs keep the other stream's work
+// off the SMs in a recovery, and the flat kernels lose 4% (FP32) to the wait
+// between their index loads and the rest (DEP = false leaves it out).
+constexpr int64_t DEP_MAX_CTAS = 2432;
+// Size that decides it for a launch of `size` CTAs of problem p.
+inline int64_t dep_size(const ProbArgs& p, int64_t size) { return p.overlap ? size : DEP_MAX_CTAS + 1; }
+
+template <class... P, class... A>
+void launch(int64_t size, void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args) {
+  cudaLaunchConfig_t cfg;
+  std::memset(&cfg, 0, sizeof(cfg));
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = size <= DEP_MAX_CTAS ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);   // errors: the callers' cudaGetLastError
 }
 
 inline unsigned lin_grid(int64_t n, int b) { return (unsigned)((n + b - 1) / b); }
@@ -3360,7 +3463,7 @@ cudaError_t launch_gs_stream(const LevelArgs& L, const ProbArgs& p, T* u, T* uI,
   if (p.grid_cap > 0) cap = std::min(cap, p.grid_cap);
   const unsigned grid = (unsigned)std::min(g.total, cap);
   ++g_kernel_launches;
-  kern<<<grid, dim3(32, STREAM_CONSUMERS + 1), smem, s>>>(L.N, L.rs, L.block, u, uI, fI, W, Winv, fv, Wv, tiles,
+  launch(dep_size(p, g.total), kern, grid, dim3(32, STREAM_CONSUMERS + 1), smem, s, L.N, L.rs, L.block, u, uI, fI, W, Winv, fv, Wv, tiles,
                                                          n_tiles, p.act, p.n_act, colour, L.cptr, L.cps, L.cp_off,
                                        p.free_if + p.col_off[colour], n, if_tab<T>(p, p.col_off[colour]),
                                        g.n_if_units, p.sched, slot, p.wait_limit, p.err);
@@ -3417,10 +3520,13 @@ cudaError_t gs_colour(const LevelArgs& L, const ProbArgs& p, T* u, T* uI, const 
     const int n_if_ctas = (int)lin_grid(n, CTA);
     const int n_vol_ctas = p.n_act > 0 ? (int)lin_grid((int64_t)n_items * p.n_act, CTA) : 0;
     if (n_if_ctas + n_vol_ctas == 0) return cudaSuccess;
-    auto kern = !seven_point ? k_gs_flat<T, false, false> : fs ? k_gs_flat<T, true, true> : k_gs_flat<T, true, false>;
+    const bool dep = dep_size(p, n_if_ctas + n_vol_ctas) <= DEP_MAX_CTAS;
+    auto kern = !seven_point ? (dep ? k_gs_flat<T, false, false, true> : k_gs_flat<T, false, false, false>)
+                : fs         ? (dep ? k_gs_flat<T, true, true, true> : k_gs_flat<T, true, true, false>)
+                             : (dep ? k_gs_flat<T, true, false, true> : k_gs_flat<T, true, false, false>);
     if (ev_begin) cudaEventRecord(ev_begin, s);
     ++g_kernel_launches;
-    kern<<<n_if_ctas + n_vol_ctas, cta_shape(), 0, s>>>(
+    launch(dep_size(p, n_if_ctas + n_vol_ctas), kern, n_if_ctas + n_vol_ctas, cta_shape(), 0, s,
         L.N, L.rs, L.block, u, uI, fI, W, Winv, fs ? fs : f, Wsc ? Wsc : W, items + off[colour], n_items, p.act,
         p.n_act, colour, L.cptr, L.cps, L.cp_off, p.free_if + p.col_off[colour], n, if_tab<T>(p, p.col_off[colour]),
         n_if_ctas, n_vol_ctas);
@@ -3433,7 +3539,7 @@ cudaError_t gs_colour(const LevelArgs& L, const ProbArgs& p, T* u, T* uI, const 
   const unsigned grid = resident_grid((const void*)kern, g.total, p.grid_cap);
   if (ev_begin) cudaEventRecord(ev_begin, s);
   ++g_kernel_launches;
-  kern<<<grid, cta_shape(), 0, s>>>(L.N, L.rs, L.block, u, uI, f, fI, W, Winv, fs, Wsc, L.tiles_int, L.n_tiles_int, p.act,
+  launch(dep_size(p, g.total), kern, grid, cta_shape(), 0, s, L.N, L.rs, L.block, u, uI, f, fI, W, Winv, fs, Wsc, L.tiles_int, L.n_tiles_int, p.act,
                                     p.n_act, colour, L.cptr, L.cps, L.cp_off, p.free_if + p.col_off[colour], n,
                                     if_tab<T>(p, p.col_off[colour]), g.n_if_units, p.sched);
   if (ev_end) cudaEventRecord(ev_end, s);
@@ -3486,8 +3592,10 @@ cudaError_t residual(const LevelArgs& L, const ProbArgs& p, const T* u, const T*
     const int n_if_chunks = (int)lin_grid(n + n_zero, CTA);
     const int n_vol_chunks = p.n_act > 0 ? (int)lin_grid((int64_t)n_items * p.n_act, CTA) : 0;
     ++g_kernel_launches;
-    auto kern = seven_point ? k_res_flat<T, true, true, false> : k_res_flat<T, false, true, false>;
-    kern<<<n_if_chunks + n_vol_chunks, cta_shape(), 0, s>>>(
+    const bool dep = dep_size(p, n_if_chunks + n_vol_chunks) <= DEP_MAX_CTAS;
+    auto kern = seven_point ? (dep ? k_res_flat<T, true, true, false, true> : k_res_flat<T, true, true, false, false>)
+                            : (dep ? k_res_flat<T, false, true, false, true> : k_res_flat<T, false, true, false, false>);
+    launch(dep_size(p, n_if_chunks + n_vol_chunks), kern, n_if_chunks + n_vol_chunks, cta_shape(), 0, s,
         L.N, L.rs, L.block, u, uI, f, fI, r, W, items, make_int4(off[0], off[1], off[2], off[3]), n_items, p.act,
         p.n_act, L.cptr, L.cps, L.cp_off, p.free_if, n, if_tab<T>(p, 0), p.zero_off, n_zero, n_if_chunks,
         n_vol_chunks, nullptr, sk, sk >= 0 ? p.col_off[sk] : 0, sk >= 0 ? p.col_off[sk + 1] : 0);
@@ -3505,7 +3613,7 @@ cudaError_t residual(const LevelArgs& L, const ProbArgs& p, const T* u, const T*
   const unsigned grid = resident_grid((const void*)kern, g.total, p.grid_cap);
   if (n_part && norm) *n_part = (int)grid;
   ++g_kernel_launches;
-  kern<<<grid, cta_shape(), 0, s>>>(L.N, L.rs, L.block, u, uI, f, fI, r, W, L.tiles_int, L.n_tiles_int, p.act,
+  launch(dep_size(p, g.total), kern, grid, cta_shape(), 0, s, L.N, L.rs, L.block, u, uI, f, fI, r, W, L.tiles_int, L.n_tiles_int, p.act,
                                     p.n_act, L.cptr, L.cps, L.cp_off, p.free_if, n, if_tab<T>(p, 0), p.zero_off, n_zero,
                                     g.n_if_units, partial, p.sched, skip >= 0 && skip < 4 ? skip : -1, skip_lo, skip_hi);
   return cudaGetLastError();
@@ -3541,14 +3649,16 @@ cudaError_t restrict_to(const LevelArgs& C, const LevelArgs& F, const ProbArgs& 
     const int n_if_ctas = (int)lin_grid(n + pc.n_zero, CTA);
     const int n_vol_ctas = pc.n_act > 0 ? (int)lin_grid((int64_t)C.n_slots * pc.n_act, CTA) : 0;
     ++g_kernel_launches;
-    k_restrict_flat<T><<<n_if_ctas + n_vol_ctas, cta_shape(), 0, s>>>(
+    const int64_t size = dep_size(pc, n_if_ctas + n_vol_ctas);
+    auto kern = size <= DEP_MAX_CTAS ? k_restrict_flat<T, true> : k_restrict_flat<T, false>;
+    launch(size, kern, n_if_ctas + n_vol_ctas, cta_shape(), 0, s,
         C.N, C.rs, C.block, fc, fIc, uc, uIc, F.N, F.rs, F.block, rf, C.slot_items, C.n_slots, pc.act, pc.n_act,
         C.cptr, C.cps, C.cp_off, pc.free_if, n, pc.gather, pc.zero_off, pc.n_zero, n_if_ctas, n_vol_ctas);
     return cudaGetLastError();
   }
   const unsigned grid = resident_grid((const void*)k_restrict<T>, g.total, pc.grid_cap);
   ++g_kernel_launches;
-  k_restrict<T><<<grid, cta_shape(), 0, s>>>(C.N, C.rs, C.block, fc, fIc, uc, uIc, F.N, F.rs, F.block, rf, C.tiles_int,
+  launch(dep_size(pc, g.total), k_restrict<T>, grid, cta_shape(), 0, s, C.N, C.rs, C.block, fc, fIc, uc, uIc, F.N, F.rs, F.block, rf, C.tiles_int,
                                              C.n_tiles_int, pc.act, pc.n_act, C.cptr, C.cps, C.cp_off, pc.free_if, n,
                                              pc.gather, pc.zero_off, pc.n_zero, g.n_if_units, pc.sched);
   return cudaGetLastError();
@@ -3597,7 +3707,9 @@ cudaError_t prolong_add(const LevelArgs& F, const LevelArgs& C, const ProbArgs& 
     const int n_if_ctas = (int)lin_grid(n, CTA);
     const int n_vol_ctas = pf.n_act > 0 ? (int)lin_grid((int64_t)n_items * pf.n_act, CTA) : 0;
     ++g_kernel_launches;
-    k_prolong_flat<T><<<n_if_ctas + n_vol_ctas, cta_shape(), 0, s>>>(
+    const int64_t size = dep_size(pf, n_if_ctas + n_vol_ctas);
+    auto kern = size <= DEP_MAX_CTAS ? k_prolong_flat<T, true> : k_prolong_flat<T, false>;
+    launch(size, kern, n_if_ctas + n_vol_ctas, cta_shape(), 0, s,
         F.N, F.rs, F.block, uf, uIf, C.N, C.rs, C.block, uc, items + off[first_c], n_items, first_c,
         make_int3(rel[0], rel[1], rel[2]), pf.act,
         pf.n_act, F.cptr, F.cps, F.cp_off, pf.free_if, n, if_lo, if_hi, n_if_ctas, n_vol_ctas);
@@ -3605,7 +3717,7 @@ cudaError_t prolong_add(const LevelArgs& F, const LevelArgs& C, const ProbArgs& 
   }
   const unsigned grid = resident_grid((const void*)k_prolong<T>, g.total, pf.grid_cap);
   ++g_kernel_launches;
-  k_prolong<T><<<grid, cta_shape(), 0, s>>>(F.N, F.rs, F.block, uf, uIf, C.N, C.rs, C.block, uc, F.tiles_int,
+  launch(dep_size(pf, g.total), k_prolong<T>, grid, cta_shape(), 0, s, F.N, F.rs, F.block, uf, uIf, C.N, C.rs, C.block, uc, F.tiles_int,
                                             F.n_tiles_int, pf.act, pf.n_act, F.cptr, F.cps, F.cp_off, pf.free_if, n,
                                             g.n_if_units, pf.sched, skip, if_lo, if_hi);
   return cudaGetLastError();
@@ -3757,12 +3869,14 @@ cudaError_t coarse_cg(const DevProblem& p, const T* f, const T* fI, T* u, T* uI,
     cfg.blockDim = dim3(32 * (sh.warps + 1));   // and the scalar warp
     cfg.dynamicSmemBytes = sh.smem;
     cfg.stream = s;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = sh.ctas;
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = p.overlap ? 2 : 1;
     ++g_kernel_launches;
     const auto kern = sh.blocks_per_warp == 0 ? k_cg_cluster<T, 0, 0, false>
                       : dinv                  ? cg_kernel<T, true>(sh, A.K)
@@ -3770,7 +3884,7 @@ cudaError_t coarse_cg(const DevProblem& p, const T* f, const T* fI, T* u, T* uI,
     return cudaLaunchKernelEx(&cfg, kern, A, f, fI, u, uI);
   }
   ++g_kernel_launches;
-  k_cg<T><<<1, CG_THREADS, 0, s>>>(p.n_cg, p.rowptr, p.col, p.val, p.fsrc, f, fI, p.uptr, p.udst, p.umaster, u, uI,
+  launch(p.overlap ? 1 : DEP_MAX_CTAS + 1, k_cg<T>, 1, CG_THREADS, 0, s, p.n_cg, p.rowptr, p.col, p.val, p.fsrc, f, fI, p.uptr, p.udst, p.umaster, u, uI,
                                    work ? work : p.cg_work, dinv, rtol, maxit, p.cg_iters);
   return cudaGetLastError();
 }
@@ -3784,7 +3898,7 @@ cudaError_t fma_probe(double* out, int blocks, int iters, cudaStream_t s) {
 cudaError_t reduce_partials(const double* partial, int n, double* out, cudaStream_t s) {
   if (g_rec) return cudaSuccess;   // a batch needs no norms
   ++g_kernel_launches;
-  k_reduce<<<1, 1024, 0, s>>>(partial, n, out);
+  launch(1, k_reduce, 1, 1024, 0, s, partial, n, out);
   return cudaGetLastError();
 }
 
@@ -3796,7 +3910,7 @@ cudaError_t import_vec(const LevelArgs& L, const MacroGeo* geo, int n_macro, int
   // filters to the interior)
   if (L.n_tiles_all > 0) {
     ++g_kernel_launches;
-    k_import_vol<T><<<dim3((unsigned)L.n_tiles_all, (unsigned)n_macro), cta_shape(), 0, s>>>(
+    launch((int64_t)L.n_tiles_all * n_macro, k_import_vol<T>, dim3((unsigned)L.n_tiles_all, (unsigned)n_macro), cta_shape(), 0, s,
         L.N, L.rs, L.block, geo, nx, ny, g, blocks, L.tiles_all, closed);
   }
   return cudaGetLastError();
@@ -3808,7 +3922,7 @@ cudaError_t export_vec(const LevelArgs& L, const MacroGeo* geo, int n_macro, int
   (void)masters;
   if (L.n_tiles_all > 0) {
     ++g_kernel_launches;
-    k_export_vol<T><<<dim3((unsigned)L.n_tiles_all, (unsigned)n_macro), cta_shape(), 0, s>>>(
+    launch((int64_t)L.n_tiles_all * n_macro, k_export_vol<T>, dim3((unsigned)L.n_tiles_all, (unsigned)n_macro), cta_shape(), 0, s,
         L.N, L.rs, L.block, geo, nx, ny, blocks, g, L.tiles_all);
   }
   return cudaGetLastError();
@@ -3818,7 +3932,7 @@ template <class T>
 cudaError_t import_masters(const int64_t* gid, int n, const double* g, T* m, cudaStream_t s) {
   if (n > 0) {
     ++g_kernel_launches;
-    k_import_if<T><<<lin_grid(n, 256), 256, 0, s>>>(gid, n, g, m);
+    launch(lin_grid(n, 256), k_import_if<T>, lin_grid(n, 256), 256, 0, s, gid, n, g, m);
   }
   return cudaGetLastError();
 }
@@ -3827,7 +3941,7 @@ template <class T>
 cudaError_t export_masters(const int64_t* gid, int n, const T* m, double* g, cudaStream_t s) {
   if (n > 0) {
     ++g_kernel_launches;
-    k_export_if<T><<<lin_grid(n, 256), 256, 0, s>>>(gid, n, m, g);
+    launch(lin_grid(n, 256), k_export_if<T>, lin_grid(n, 256), 256, 0, s, gid, n, m, g);
   }
   return cudaGetLastError();
 }
@@ -3836,7 +3950,7 @@ cudaError_t grad_partials(const LevelArgs& L, int n_macro, const double* u, cons
                           double* partial, cudaStream_t s) {
   if (L.n_tiles_all > 0 && n_macro > 0) {
     ++g_kernel_launches;
-    k_grad<<<dim3((unsigned)L.n_tiles_all, (unsigned)n_macro), cta_shape(), 0, s>>>(L.N, L.rs, L.block, u, lam, W,
+    launch((int64_t)L.n_tiles_all * n_macro, k_grad, dim3((unsigned)L.n_tiles_all, (unsigned)n_macro), cta_shape(), 0, s, L.N, L.rs, L.block, u, lam, W,
                                                                                    L.tiles_all, partial);
   }
   return cudaGetLastError();
@@ -3845,7 +3959,7 @@ cudaError_t grad_partials(const LevelArgs& L, int n_macro, const double* u, cons
 cudaError_t reduce_per_macro(const double* partial, int n_per, int n_macro, double* out, cudaStream_t s) {
   if (n_macro > 0) {
     ++g_kernel_launches;
-    k_reduce_per_macro<<<n_macro, 256, 0, s>>>(partial, n_per, out);
+    launch(n_macro, k_reduce_per_macro, n_macro, 256, 0, s, partial, n_per, out);
   }
   return cudaGetLastError();
 }
@@ -3855,9 +3969,9 @@ cudaError_t apply_if_nodes(const LevelArgs& L, const double* u, const double* uI
   if (n > 0) {
     ++g_kernel_launches;
     if (seven_point)
-      k_if_apply<true><<<lin_grid(n, 128), 128, 0, s>>>(L.N, L.rs, L.block, u, uI, W, L.cptr, L.cps, list, n, out);
+      launch(lin_grid(n, 128), k_if_apply<true>, lin_grid(n, 128), 128, 0, s, L.N, L.rs, L.block, u, uI, W, L.cptr, L.cps, list, n, out);
     else
-      k_if_apply<false><<<lin_grid(n, 128), 128, 0, s>>>(L.N, L.rs, L.block, u, uI, W, L.cptr, L.cps, list, n, out);
+      launch(lin_grid(n, 128), k_if_apply<false>, lin_grid(n, 128), 128, 0, s, L.N, L.rs, L.block, u, uI, W, L.cptr, L.cps, list, n, out);
   }
   return cudaGetLastError();
 }
@@ -3865,7 +3979,7 @@ cudaError_t apply_if_nodes(const LevelArgs& L, const double* u, const double* uI
 cudaError_t copy_listed(const double* src, double* dst, const int* idx, int n, cudaStream_t s) {
   if (n > 0) {
     ++g_kernel_launches;
-    k_copy_listed<<<lin_grid(n, 256), 256, 0, s>>>(src, dst, idx, n);
+    launch(lin_grid(n, 256), k_copy_listed, lin_grid(n, 256), 256, 0, s, src, dst, idx, n);
   }
   return cudaGetLastError();
 }
@@ -3883,7 +3997,7 @@ cudaError_t set_masters_zero(double* uI, const int* ids, int n, cudaStream_t s) 
   }
   if (n > 0) {
     ++g_kernel_launches;
-    k_set_masters_zero<<<lin_grid(n, 256), 256, 0, s>>>(uI, ids, n);
+    launch(lin_grid(n, 256), k_set_masters_zero, lin_grid(n, 256), 256, 0, s, uI, ids, n);
   }
   return cudaGetLastError();
 }
@@ -3893,7 +4007,7 @@ cudaError_t scale_blocks(const double* f, const double* winv, double* out, int n
   const int64_t total = (int64_t)n_macro * block;
   if (total > 0) {
     ++g_kernel_launches;
-    k_scale_blocks<<<(unsigned)std::min<int64_t>(lin_grid(total, 256), 152 * 16), 256, 0, s>>>(f, winv, out, n_macro,
+    launch(lin_grid(total, 256), k_scale_blocks, (unsigned)std::min<int64_t>(lin_grid(total, 256), 152 * 16), 256, 0, s, f, winv, out, n_macro,
                                                                                                block);
   }
   return cudaGetLastError();
@@ -3914,7 +4028,7 @@ cudaError_t restore_copies(double* u, const double* uI, const int64_t* off, cons
   }
   if (n > 0) {
     ++g_kernel_launches;
-    k_restore<<<lin_grid(n, 256), 256, 0, s>>>(u, uI, off, master, n);
+    launch(lin_grid(n, 256), k_restore, lin_grid(n, 256), 256, 0, s, u, uI, off, master, n);
   }
   return cudaGetLastError();
 }
@@ -3952,7 +4066,7 @@ cudaError_t residual_to_f32(const LevelArgs& L, const ProbArgs& p, const double*
   const unsigned grid = resident_grid((const void*)kern, g.total, p.grid_cap);
   if (n_part) *n_part = (int)grid;
   ++g_kernel_launches;
-  kern<<<grid, cta_shape(), 0, s>>>(L.N, L.rs, L.block, u, uI, f, fI, f32, fI32, W, L.tiles_int, L.n_tiles_int, p.act,
+  launch(dep_size(p, g.total), kern, grid, cta_shape(), 0, s, L.N, L.rs, L.block, u, uI, f, fI, f32, fI32, W, L.tiles_int, L.n_tiles_int, p.act,
                                     p.n_act, L.cptr, L.cps, p.free_if, n, if_tab<double>(p, 0), g.n_if_units, partial,
                                     p.sched);
   return cudaGetLastError();
@@ -3985,12 +4099,12 @@ cudaError_t add_correction(const LevelArgs& L, const ProbArgs& p, double* u, dou
     const int64_t per = 256 * 8;
     const unsigned gx = (unsigned)std::min<int64_t>((L.block / 2 + per - 1) / per, 4096);
     ++g_kernel_launches;
-    k_add_corr_blocks<<<dim3(gx, (unsigned)p.n_act), 256, 0, s>>>(u, e, L.block, p.act);
+    launch(dep_size(p, (int64_t)gx * p.n_act), k_add_corr_blocks, dim3(gx, (unsigned)p.n_act), 256, 0, s, u, e, L.block, p.act);
   }
   const int n = p.col_off[4];
   if (n > 0) {
     ++g_kernel_launches;
-    k_add_corr_masters<<<lin_grid(n, 256), 256, 0, s>>>(uI, eI, p.free_if, n);
+    launch(dep_size(p, lin_grid(n, 256)), k_add_corr_masters, lin_grid(n, 256), 256, 0, s, uI, eI, p.free_if, n);
   }
   return cudaGetLastError();
 }
@@ -4020,12 +4134,12 @@ cudaError_t zero_problem_blocks(const LevelArgs& L, const ProbArgs& p, T* u, T* 
     const int64_t per = 256 * 8;
     unsigned gx = (unsigned)std::min<int64_t>((L.block + per - 1) / per, 4096);
     ++g_kernel_launches;
-    k_zero_blocks<T><<<dim3(gx, p.n_act), 256, 0, s>>>(u, L.block, p.act);
+    launch(dep_size(p, (int64_t)gx * p.n_act), k_zero_blocks<T>, dim3(gx, p.n_act), 256, 0, s, u, L.block, p.act);
   }
   const int n = p.col_off[4];
   if (n > 0) {
     ++g_kernel_launches;
-    k_zero_list<T><<<lin_grid(n, 256), 256, 0, s>>>(uI, p.free_if, n);
+    launch(dep_size(p, lin_grid(n, 256)), k_zero_list<T>, lin_grid(n, 256), 256, 0, s, uI, p.free_if, n);
   }
   return cudaGetLastError();
 }
