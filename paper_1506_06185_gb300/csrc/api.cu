@@ -72,6 +72,13 @@ struct Prec {
 
 }  // namespace
 
+// Shared by a mesh and the batches that hold its buffers, so that either may be
+// destroyed first.
+struct MeshRefs {
+  int batches = 0;     // batches that hold the mesh's buffers
+  bool alive = true;   // the mesh has not been destroyed
+};
+
 struct hhg_mesh {
   HostMesh host;
   int device = 0;
@@ -133,7 +140,7 @@ struct hhg_mesh {
   // when another set replaces it; `collect`, when set, receives new ones
   std::vector<void*> fault_allocs, dn_allocs;
   std::vector<void*>* collect = nullptr;
-  int batch_refs = 0;              // batch graphs that hold this mesh's buffers
+  std::shared_ptr<MeshRefs> refs = std::make_shared<MeshRefs>();
   int64_t bytes = 0;
   double* host_scalar = nullptr;   // pinned
   double* grad_partial = nullptr;  // coefficient-gradient partial sums
@@ -166,6 +173,7 @@ struct hhg_batch {
     cudaStream_t stream;
     cudaEvent_t done;       // join dependency inside the capture
     cudaEvent_t done_time;  // event-record node: completion time of the task
+    std::shared_ptr<MeshRefs> refs;
   };
   std::vector<Task> tasks;       // recovery tasks, then (optionally) the global one
   bool mixed = false;
@@ -215,7 +223,7 @@ int dalloc(hhg_mesh* m, T** p, size_t n) {
 // batch graph still refers to the mesh's buffers (then they stay until the
 // mesh is destroyed).
 void release(hhg_mesh* m, std::vector<void*>& list) {
-  if (m->batch_refs > 0) {
+  if (m->refs->batches > 0) {
     list.clear();
     return;
   }
@@ -1378,6 +1386,13 @@ int upload_priorities(hhg_batch* b, const std::vector<int>& prio) {
 }
 
 // Records every task's program and uploads it with the scheduler's counters.
+// The batch's device is current and its meshes are still there.
+int check_batch(const hhg_batch* b) {
+  for (const auto& t : b->tasks)
+    if (t.refs && !t.refs->alive) return fail(HHG_ERR_STATE, "a mesh of the batch has been destroyed");
+  return b->tasks.empty() ? HHG_OK : check_device(b->tasks[0].mesh);
+}
+
 int setup_persistent(hhg_batch* b, size_t n_rec) {
   b->op_off.assign(1, 0);
   for (size_t t = 0; t < b->tasks.size(); ++t) {
@@ -1635,6 +1650,7 @@ int hhg_mesh_destroy(hhg_mesh* m) {
   for (cudaEvent_t ev : m->prof_ev) cudaEventDestroy(ev);
   for (cudaEvent_t ev : m->bd_ev) cudaEventDestroy(ev);
   const int dev = m->device;
+  m->refs->alive = false;
   delete m;
   if (cur >= 0 && cur != dev) cudaSetDevice(cur);
   return HHG_OK;
@@ -1925,14 +1941,17 @@ int hhg_batch_create(hhg_mesh* global, int global_cycles, hhg_mesh* const* meshe
     return cleanup(rc);
   }
   // the graph holds the meshes' buffers: a new fault set may not free them
-  for (auto& t : b->tasks) ++t.mesh->batch_refs;
+  for (auto& t : b->tasks) {
+    t.refs = t.mesh->refs;
+    ++t.refs->batches;
+  }
   *out = b.release();
   return HHG_OK;
 }
 
 int hhg_batch_launch(hhg_batch* b, double* task_ms, void* stream) {
   if (!b) return fail(HHG_ERR_ARG, "null batch");
-  if (!b->tasks.empty()) HHG_TRY(check_device(b->tasks[0].mesh));
+  HHG_TRY(check_batch(b));
   cudaStream_t s = (cudaStream_t)stream;
   HHG_CUDA(cudaGraphLaunch(b->exec, s));
   g_kernel_launches += b->kernels;
@@ -1950,7 +1969,7 @@ int hhg_batch_launch(hhg_batch* b, double* task_ms, void* stream) {
 int hhg_batch_launch_persistent(hhg_batch* b, double* task_ms, void* stream) {
   if (!b) return fail(HHG_ERR_ARG, "null batch");
   if (b->tasks.empty()) return HHG_OK;
-  HHG_TRY(check_device(b->tasks[0].mesh));
+  HHG_TRY(check_batch(b));
   cudaStream_t s = (cudaStream_t)stream;
   const int n = (int)b->tasks.size();
   const int n_ops = (int)b->ops.size();
@@ -1986,7 +2005,7 @@ int hhg_batch_launch_persistent(hhg_batch* b, double* task_ms, void* stream) {
 int hhg_batch_set_priority(hhg_batch* b, const int* prio) {
   if (!b) return fail(HHG_ERR_ARG, "null batch");
   if (b->tasks.empty()) return HHG_OK;
-  HHG_TRY(check_device(b->tasks[0].mesh));
+  HHG_TRY(check_batch(b));
   std::vector<int> p(b->tasks.size(), 0);
   if (prio) p.assign(prio, prio + b->tasks.size());
   HHG_CUDA(cudaDeviceSynchronize());   // no launch may still read the old order
@@ -2011,7 +2030,7 @@ int hhg_batch_destroy(hhg_batch* b) {
   if (b->exec) cudaGraphExecDestroy(b->exec);
   if (b->graph) cudaGraphDestroy(b->graph);
   for (auto& t : b->tasks) {
-    --t.mesh->batch_refs;
+    if (t.refs) --t.refs->batches;
     if (t.stream) cudaStreamDestroy(t.stream);
     if (t.done) cudaEventDestroy(t.done);
     if (t.done_time) cudaEventDestroy(t.done_time);
