@@ -451,8 +451,8 @@ int hhg_set_streaming(hhg_mesh* mesh, int enable);
  * level.  On those levels the residual before each restriction, the
  * restriction onto the level (one thread per slot of four coarse nodes) and
  * the prolongation onto it (one thread per 16-byte vector of same-colour fine
- * nodes) run in the same flat form; the stopping test's norm keeps the tile
- * kernel.  Same iterate bit for bit as the tile kernels.  The streaming kernel
+ * nodes) run in the same flat form; the stopping test's norm runs flat up
+ * to 16384 CTAs and in the tile kernel beyond.  Same iterate bit for bit as the tile kernels.  The streaming kernel
  * (hhg_set_streaming) takes precedence where both are enabled; the
  * persistent batch executor keeps the tile kernel.  Drops the captured
  * recovery-cycle graph. */

@@ -462,7 +462,7 @@ int upload_problem(hhg_mesh* m, const HostProblem& h, DevProblem& d) {
   HHG_TRY(dalloc(m, &d.cg_dinv_buf, (size_t)std::max(1, h.n_cg)));
   HHG_TRY(upload_diagonal(h, d));
   const int L = (int)m->host.lv.size() - 1;
-  d.n_partial = m->tab[L].n_tiles_int * std::max(1, d.n_act) + (m->host.lv[L].n_if + 127) / 128 + 64;
+  d.n_partial = std::max(FLAT_NORM_MAX, m->tab[L].n_tiles_int * std::max(1, d.n_act) + (m->host.lv[L].n_if + 127) / 128 + 64);
   HHG_TRY(dalloc(m, &d.partial, (size_t)d.n_partial));
   HHG_TRY(dalloc(m, &d.scalar, 8));
   HHG_TRY(dalloc(m, &d.cg_iters, 4));
@@ -696,20 +696,20 @@ int norm2_async(hhg_mesh* m, DevProblem& p, cudaStream_t s, bool after_smoothing
   const int skip = after_smoothing && !m->host.general ? 3 : -1;
   HHG_CUDA(residual<double>(plargs(m, p, L), pargs(p, L), D.u, D.uI, D.f, level_fI<double>(D, p, true), nullptr, D.W,
                             m->host.seven_point, false, p.partial, &np, s, skip));
-  HHG_CUDA(reduce_partials(p.partial, np, p.scalar, s));
+  const bool read = p.kind == 0;   // the one whose norm the host reads
+  HHG_CUDA(reduce_partials(p.partial, np, p.scalar, s, read ? m->host_scalar : nullptr, m->dev_err,
+                           read ? m->host_flag : nullptr));
   return HHG_OK;
 }
 
-// Reads a device scalar (synchronising s) together with the mesh's error
+// Waits for s and reads the squared norm that the last reduce_partials of the
+// global problem on s left in pinned memory, together with the mesh's error
 // flag; a set flag (a bounded device wait ran out in an earlier kernel) is
 // cleared and reported as HHG_ERR_TIMEOUT.
-int read_scalar(hhg_mesh* m, const double* dev, double* out, cudaStream_t s) {
-  HHG_CUDA(cudaMemcpyAsync(m->host_scalar, dev, sizeof(double), cudaMemcpyDeviceToHost, s));
-  HHG_CUDA(cudaMemcpyAsync(m->host_flag, m->dev_err, sizeof(int), cudaMemcpyDeviceToHost, s));
+int read_norm2(hhg_mesh* m, double* out, cudaStream_t s) {
   HHG_CUDA(cudaStreamSynchronize(s));
-  *out = *m->host_scalar;
-  if (*m->host_flag != 0) {
-    const int code = *m->host_flag;
+  *out = *(volatile double*)m->host_scalar;
+  if (const int code = *(volatile int*)m->host_flag; code != 0) {
     HHG_CUDA(cudaMemsetAsync(m->dev_err, 0, sizeof(int), s));
     HHG_CUDA(cudaStreamSynchronize(s));
     return fail(HHG_ERR_TIMEOUT, code == 1 ? "a bounded device wait ran out (the iterate is incomplete)"
@@ -721,7 +721,7 @@ int read_scalar(hhg_mesh* m, const double* dev, double* out, cudaStream_t s) {
 int resnorm(hhg_mesh* m, double* out, cudaStream_t s) {
   HHG_TRY(norm2_async(m, m->global, s));
   double v = 0.0;
-  HHG_TRY(read_scalar(m, m->global.scalar, &v, s));
+  HHG_TRY(read_norm2(m, &v, s));
   *out = std::sqrt(v);
   return HHG_OK;
 }
@@ -738,7 +738,9 @@ int ir_residual(hhg_mesh* m, DevProblem& p, cudaStream_t s) {
   int np = 0;
   HHG_CUDA(residual_to_f32(plargs(m, p, L), pargs(p, L), D.u, D.uI, D.f, level_fI<double>(D, p, true), E.f, E.fI, D.W,
                            m->host.seven_point, p.partial, &np, s));
-  HHG_CUDA(reduce_partials(p.partial, np, p.scalar, s));
+  const bool read = p.kind == 0;   // the one whose norm the host reads
+  HHG_CUDA(reduce_partials(p.partial, np, p.scalar, s, read ? m->host_scalar : nullptr, m->dev_err,
+                           read ? m->host_flag : nullptr));
   return HHG_OK;
 }
 
@@ -1678,28 +1680,36 @@ int hhg_set_problem(hhg_mesh* m, const double* f, const double* u0, void* stream
   const LevelArgs a = largs(m, L);
   DevLevel<double>& D = m->d64.lv[L];
   int rc;
-  const bool gen = m->host.general;
-  const int64_t n_if = m->host.lv[L].n_if;
+  const int n_if = m->host.lv[L].n_if;
+  if (!m->host.general) {
+    // both vectors in one launch, unless they pass through the staging buffer
+    const double* gf = f ? stage_in(m, f, s, &rc) : nullptr;
+    if (f && !gf) return rc;
+    auto import = [&](const double* vf, const double* vu) {
+      return import_problem(a, m->geo, m->host.n_macro, m->host.nx, m->host.ny, vf, vu, D.f, m->fs_top,
+                            m->d64.Winv[L], D.u, a.if_gid, n_if, D.fI, D.uI, s);
+    };
+    if (gf && gf != f) {
+      HHG_CUDA(import(gf, nullptr));
+      gf = nullptr;
+    }
+    const double* gu = u0 ? stage_in(m, u0, s, &rc) : nullptr;
+    if (u0 && !gu) return rc;
+    if (gf || gu) HHG_CUDA(import(gf, gu));
+    return HHG_OK;
+  }
   if (f) {
     const double* g = stage_in(m, f, s, &rc);
     if (!g) return rc;
-    if (gen) HHG_CUDA(general_import_vol<double>(a, m->host.n_macro, n_if, g, D.f, s));
-    else HHG_CUDA(import_vec<double>(a, m->geo, m->host.n_macro, m->host.nx, m->host.ny, g, D.f, D.fI, false, s));
-    HHG_CUDA(import_masters<double>(a.if_gid, m->host.lv[L].n_if, g, D.fI, s));
-    if (m->fs_top)
-      HHG_CUDA(scale_blocks(D.f, m->d64.Winv[L], m->fs_top, m->host.n_macro, m->host.lv[L].block, s));
+    HHG_CUDA(general_import_vol<double>(a, m->host.n_macro, n_if, g, D.f, s));
+    HHG_CUDA(import_masters<double>(a.if_gid, n_if, g, D.fI, s));
   }
   if (u0) {
     const double* g = stage_in(m, u0, s, &rc);
     if (!g) return rc;
-    if (gen) {
-      HHG_CUDA(general_import_vol<double>(a, m->host.n_macro, n_if, g, D.u, s));
-      HHG_CUDA(import_masters<double>(a.if_gid, m->host.lv[L].n_if, g, D.uI, s));
-      HHG_CUDA(restore_copies(D.u, D.uI, m->gen_copy_off, m->gen_copy_master, m->n_gen_copy, s));
-    } else {
-      HHG_CUDA(import_vec<double>(a, m->geo, m->host.n_macro, m->host.nx, m->host.ny, g, D.u, D.uI, true, s));
-      HHG_CUDA(import_masters<double>(a.if_gid, m->host.lv[L].n_if, g, D.uI, s));
-    }
+    HHG_CUDA(general_import_vol<double>(a, m->host.n_macro, n_if, g, D.u, s));
+    HHG_CUDA(import_masters<double>(a.if_gid, n_if, g, D.uI, s));
+    HHG_CUDA(restore_copies(D.u, D.uI, m->gen_copy_off, m->gen_copy_master, m->n_gen_copy, s));
   }
   return HHG_OK;
 }
@@ -1721,11 +1731,13 @@ int hhg_get_solution(hhg_mesh* m, double* u, void* stream) {
     if (!m->staging) HHG_TRY(dalloc(m, &m->staging, (size_t)n));
     g = m->staging;
   }
-  if (m->host.general)
+  if (m->host.general) {
     HHG_CUDA(general_export_vol<double>(a, m->host.n_macro, m->host.lv[L].n_if, D.u, g, s));
-  else
-    HHG_CUDA(export_vec<double>(a, m->geo, m->host.n_macro, m->host.nx, m->host.ny, D.u, D.uI, g, s));
-  HHG_CUDA(export_masters<double>(a.if_gid, m->host.lv[L].n_if, D.uI, g, s));
+    HHG_CUDA(export_masters<double>(a.if_gid, m->host.lv[L].n_if, D.uI, g, s));
+  } else {
+    HHG_CUDA(export_solution(a, m->geo, m->host.n_macro, m->host.nx, m->host.ny, D.u, D.uI, a.if_gid,
+                             m->host.lv[L].n_if, g, s));
+  }
   if (!dev) {
     HHG_CUDA(cudaMemcpyAsync(u, g, (size_t)n * sizeof(double), cudaMemcpyDefault, s));
     HHG_CUDA(cudaStreamSynchronize(s));
@@ -1811,11 +1823,12 @@ int hhg_grad_coeff(hhg_mesh* m, const double* u, const double* lam, double* grad
   int rc;
   const double* g = stage_in(m, u, s, &rc);
   if (!g) return rc;
-  HHG_CUDA(import_vec<double>(a, m->geo, n_macro, m->host.nx, m->host.ny, g, D.u, D.uI, true, s));
-  HHG_CUDA(import_masters<double>(a.if_gid, m->host.lv[L].n_if, g, D.uI, s));
+  HHG_CUDA(import_problem(a, m->geo, n_macro, m->host.nx, m->host.ny, nullptr, g, nullptr, nullptr, nullptr, D.u,
+                          a.if_gid, m->host.lv[L].n_if, nullptr, D.uI, s));
   const double* gl = stage_in(m, lam, s, &rc);
   if (!gl) return rc;
-  HHG_CUDA(import_vec<double>(a, m->geo, n_macro, m->host.nx, m->host.ny, gl, D.r, nullptr, true, s));
+  HHG_CUDA(import_problem(a, m->geo, n_macro, m->host.nx, m->host.ny, nullptr, gl, nullptr, nullptr, nullptr, D.r,
+                          a.if_gid, 0, nullptr, nullptr, s));
   HHG_CUDA(grad_partials(a, n_macro, D.u, D.r, D.W, m->grad_partial, s));
   HHG_CUDA(reduce_per_macro(m->grad_partial, a.n_tiles_all, n_macro, m->grad_out, s));
   std::vector<double> out(n_macro);
@@ -2227,7 +2240,7 @@ int hhg_solve(hhg_mesh* m, const hhg_solve_opts* o, double* hist, int* n_hist, i
   double r0 = 0.0, v = 0.0;
   if (mixed) {
     HHG_TRY(ir_residual(m, m->global, s));
-    HHG_TRY(read_scalar(m, m->global.scalar, &v, s));
+    HHG_TRY(read_norm2(m, &v, s));
     r0 = std::sqrt(v);
   } else {
     HHG_TRY(resnorm(m, &r0, s));
@@ -2249,13 +2262,13 @@ int hhg_solve(hhg_mesh* m, const hhg_solve_opts* o, double* hist, int* n_hist, i
       HHG_TRY(bd_mark(m, s, BD_NORM));
       HHG_TRY(ir_residual(m, m->global, s));
       HHG_TRY(bd_mark(m, s, BD_HOST));
-      HHG_TRY(read_scalar(m, m->global.scalar, &v, s));
+      HHG_TRY(read_norm2(m, &v, s));
     } else {
       HHG_TRY(vcycle_T<double>(m, m->d64, m->global, pre, post, cg_rtol, cg_maxit, s));
       HHG_TRY(bd_mark(m, s, BD_NORM));
       HHG_TRY(norm2_async(m, m->global, s, post > 0));
       HHG_TRY(bd_mark(m, s, BD_HOST));
-      HHG_TRY(read_scalar(m, m->global.scalar, &v, s));
+      HHG_TRY(read_norm2(m, &v, s));
     }
     ++k;
     rel = r0 > 0 ? std::sqrt(v) / r0 : 0.0;
@@ -2278,7 +2291,7 @@ int hhg_solve(hhg_mesh* m, const hhg_solve_opts* o, double* hist, int* n_hist, i
       if (mixed) HHG_TRY(ir_residual(m, m->global, s));
       else HHG_TRY(norm2_async(m, m->global, s));
       HHG_TRY(bd_mark(m, s, BD_HOST));
-      HHG_TRY(read_scalar(m, m->global.scalar, &v, s));
+      HHG_TRY(read_norm2(m, &v, s));
       rel = r0 > 0 ? std::sqrt(v) / r0 : 0.0;
       push(rel);
     }

@@ -340,6 +340,11 @@ struct DevLevel {
   T* W = nullptr;   // [n_macro][16][15]
 };
 
+// CTAs of a residual norm at most that run in the flat form (norm and read-back
+// at 29791 nodes 30 -> 24 us, 1.6e6 nodes 78 -> 57 us, 7.2e6 nodes (11000 CTAs)
+// 231 -> 181 us, 15-point 397 -> 283 us; at 1.3e8 nodes the tile form is 12%
+// faster, its CTAs adding up many tiles each).
+constexpr int FLAT_NORM_MAX = 16384;
 // Whether a level runs the flat kernels: off, switched on, or by default (new
 // meshes, every level the kernels can run; a launch limit selects the tile
 // kernels there).

@@ -113,20 +113,22 @@ template <class T>
 cudaError_t coarse_cg(const DevProblem& p, const T* f, const T* fI, T* u, T* uI, double rtol, int maxit,
                       cudaStream_t s, double* work = nullptr);
 
-cudaError_t reduce_partials(const double* partial, int n, double* out, cudaStream_t s);
+// host, host_err (pinned host memory, may be null): also receive the sum and *err.
+cudaError_t reduce_partials(const double* partial, int n, double* out, cudaStream_t s, double* host = nullptr,
+                            const int* err = nullptr, int* host_err = nullptr);
 
 // FP64 FMA throughput probe: `blocks` CTAs of 256 threads, 8 x iters FMAs per
 // thread; out holds blocks * 256 doubles.
 cudaError_t fma_probe(double* out, int blocks, int iters, cudaStream_t s);
 
-// Global vector <-> blocked storage of one level.
-template <class T>
-cudaError_t import_vec(const LevelArgs& L, const MacroGeo* geo, int n_macro, int64_t nx, int64_t ny,
-                       const double* g, T* blocks, T* masters, bool closed, cudaStream_t s);
-template <class T>
-cudaError_t export_vec(const LevelArgs& L, const MacroGeo* geo, int n_macro, int64_t nx, int64_t ny,
-                       const T* blocks, const T* masters, double* g, cudaStream_t s);
-
+// Global vectors <-> blocked storage of one level and its masters.  Either of
+// gf, gu may be null; fs (may be null): f times the macro's winv.
+cudaError_t import_problem(const LevelArgs& L, const MacroGeo* geo, int n_macro, int64_t nx, int64_t ny,
+                           const double* gf, const double* gu, double* f, double* fs, const double* winv, double* u,
+                           const int64_t* if_gid, int n_if, double* fI, double* uI, cudaStream_t s);
+cudaError_t export_solution(const LevelArgs& L, const MacroGeo* geo, int n_macro, int64_t nx, int64_t ny,
+                            const double* u, const double* uI, const int64_t* if_gid, int n_if, double* g,
+                            cudaStream_t s);
 template <class T>
 cudaError_t import_masters(const int64_t* gid, int n, const double* g, T* m, cudaStream_t s);
 template <class T>

@@ -2507,14 +2507,24 @@ __global__ void k_reduce_per_macro(const double* __restrict__ partial, int n_per
   if (threadIdx.x == 0) out[blockIdx.x] = s;
 }
 
-__global__ void k_reduce(const double* __restrict__ partial, int n, double* __restrict__ out) {
+// Sum of the partial sums into out and, where host is given, into pinned host
+// memory with the mesh's error flag beside it: the caller waits for the stream
+// and reads them, without two copies of a few bytes behind the kernel.
+__global__ void k_reduce(const double* __restrict__ partial, int n, double* __restrict__ out, double* host,
+                         const int* __restrict__ err, int* host_err) {
   launch_next();
   after_previous();
   __shared__ double sh[33];
   double s = 0.0;
   for (int q = threadIdx.x; q < n; q += blockDim.x) s += partial[q];
   s = cta_sum(s, sh);
-  if (threadIdx.x == 0) out[0] = s;
+  if (threadIdx.x == 0) {
+    out[0] = s;
+    if (host) {
+      *host = s;
+      *host_err = *err;
+    }
+  }
 }
 
 // FP64 FMA throughput probe (measurement support): every thread runs eight
@@ -2543,48 +2553,94 @@ __device__ __forceinline__ int64_t dev_gid(const MacroGeo& g, int N, int i, int 
   return (Z * (ny + 1) + Y) * (nx + 1) + X;
 }
 
-template <class T>
-__global__ void __launch_bounds__(CTA) k_import_vol(int N, const int* __restrict__ rs, int64_t block, const MacroGeo* __restrict__ geo,
-                                                    int64_t nx, int64_t ny, const double* __restrict__ g,
-                                                    T* __restrict__ dst, const Tile* __restrict__ tiles, bool closed) {
+// Node (i, j, k) of a macro has grid index node_gid(0, j, k) + i * gid_stride_i.
+// A tile of the closed lattice is 8 rows x 128 nodes; its rows are taken in
+// the direction (j or k) in which the grid's x grows where it does not grow with
+// i, so that the 8 rows touch the same 32-byte sectors of the grid vector.  One
+// launch takes f, its scaled copy, u and both masters: 29791 nodes 25 -> 10 us,
+// 7.2e6 nodes 235 -> 156 us, 1.35e8 nodes 2.18 -> 2.10 ms (5.4 GB: the strided
+// reads of the macros whose x grows with j or k bound it).
+struct GridRow {
+  int64_t gid0, step;   // grid index of i = 0, step per i
+  int j, k, m;          // row and this thread's slot (nodes 4 m .. 4 m + 3)
+};
+__device__ __forceinline__ bool grid_row(const Tile& t, const MacroGeo& g, int N, int64_t nx, int64_t ny, GridRow& r) {
+  const int along = t.j0 + threadIdx.y;
+  const bool by_k = g.e2[0] == 0;   // x grows with k only
+  r.j = by_k ? t.k : along;
+  r.k = by_k ? along : t.k;
+  r.m = t.m0 + threadIdx.x;
+  if (r.j + r.k > N) return false;
+  r.gid0 = dev_gid(g, N, 0, r.j, r.k, nx, ny);
+  r.step = dev_gid(g, N, 1, r.j, r.k, nx, ny) - r.gid0;
+  return true;
+}
+
+// Global vectors gf and gu (either may be null) into the blocks and masters: f
+// on the interior nodes (and, where fs is given, f times the macro's winv into
+// fs), u on the closed lattice.  The first n_if_ctas CTAs take the masters.
+__global__ void __launch_bounds__(CTA) k_import(int N, const int* __restrict__ rs, int64_t block,
+                                                const MacroGeo* __restrict__ geo, int64_t nx, int64_t ny,
+                                                const double* __restrict__ gf, const double* __restrict__ gu,
+                                                double* __restrict__ f, double* __restrict__ fs,
+                                                const double* __restrict__ winv, double* __restrict__ u,
+                                                const Tile* __restrict__ tiles, int n_tiles,
+                                                const int64_t* __restrict__ if_gid, int n_if, double* __restrict__ fI,
+                                                double* __restrict__ uI, int n_if_ctas) {
   launch_next();
   after_previous();
-  const Tile t = tiles[blockIdx.x];
-  const int macro = blockIdx.y;
-  const int k = t.k;
-  const int j = t.j0 + threadIdx.y;
-  const int m = t.m0 + threadIdx.x;
-  const MacroGeo gm = geo[macro];
-  T* b = dst + (size_t)macro * block;
-  const int lo = closed ? 0 : 1, top = closed ? N : N - 1;
-  if (j < lo) return;
+  if ((int)blockIdx.x < n_if_ctas) {
+    const int q = blockIdx.x * CTA + tid256();
+    if (q >= n_if) return;
+    const int64_t g = if_gid[q];
+    if (gf) fI[q] = gf[g];
+    if (gu) uI[q] = gu[g];
+    return;
+  }
+  const int v = blockIdx.x - n_if_ctas, macro = v / n_tiles;
+  GridRow r;
+  if (!grid_row(tiles[v - macro * n_tiles], geo[macro], N, nx, ny, r)) return;
+  const size_t b = (size_t)macro * block + row_base(rs, N, r.j, r.k) + r.m;
+  const int CS = __ldg(rs + N + 2), top = N - r.j - r.k;
+  const double w = fs ? winv[macro] : 0.0;
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
-    const int i = 4 * m + q;
-    if (i < lo || i + j + k > top) continue;
-    b[lidx32(rs, N, i, j, k)] = (T)g[dev_gid(gm, N, i, j, k, nx, ny)];
+    const int i = 4 * r.m + q;
+    if (i > top) continue;
+    const int64_t g = r.gid0 + i * r.step;
+    const size_t o = b + (size_t)((i + 2 * r.j + 3 * r.k) & 3) * CS;
+    if (gu) u[o] = gu[g];
+    if (gf && i >= 1 && r.j >= 1 && r.k >= 1 && i < top) {
+      const double x = gf[g];
+      f[o] = x;
+      if (fs) fs[o] = x * w;
+    }
   }
 }
 
-template <class T>
-__global__ void __launch_bounds__(CTA) k_export_vol(int N, const int* __restrict__ rs, int64_t block, const MacroGeo* __restrict__ geo,
-                                                    int64_t nx, int64_t ny, const T* __restrict__ src,
-                                                    double* __restrict__ g, const Tile* __restrict__ tiles) {
+// The interior nodes of the blocks and the masters into the global vector g.
+__global__ void __launch_bounds__(CTA) k_export(int N, const int* __restrict__ rs, int64_t block,
+                                                const MacroGeo* __restrict__ geo, int64_t nx, int64_t ny,
+                                                const double* __restrict__ u, const double* __restrict__ uI,
+                                                double* __restrict__ g, const Tile* __restrict__ tiles, int n_tiles,
+                                                const int64_t* __restrict__ if_gid, int n_if, int n_if_ctas) {
   launch_next();
   after_previous();
-  const Tile t = tiles[blockIdx.x];
-  const int macro = blockIdx.y;
-  const int k = t.k;
-  const int j = t.j0 + threadIdx.y;
-  const int m = t.m0 + threadIdx.x;
-  const MacroGeo gm = geo[macro];
-  const T* b = src + (size_t)macro * block;
-  if (j < 1 || k < 1) return;
+  if ((int)blockIdx.x < n_if_ctas) {
+    const int q = blockIdx.x * CTA + tid256();
+    if (q < n_if) g[if_gid[q]] = uI[q];
+    return;
+  }
+  const int v = blockIdx.x - n_if_ctas, macro = v / n_tiles;
+  GridRow r;
+  if (!grid_row(tiles[v - macro * n_tiles], geo[macro], N, nx, ny, r) || r.j < 1 || r.k < 1) return;
+  const size_t b = (size_t)macro * block + row_base(rs, N, r.j, r.k) + r.m;
+  const int CS = __ldg(rs + N + 2), top = N - r.j - r.k;
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
-    const int i = 4 * m + q;
-    if (i < 1 || i + j + k > N - 1) continue;
-    g[dev_gid(gm, N, i, j, k, nx, ny)] = (double)b[lidx32(rs, N, i, j, k)];
+    const int i = 4 * r.m + q;
+    if (i < 1 || i >= top) continue;
+    g[r.gid0 + i * r.step] = u[b + (size_t)((i + 2 * r.j + 3 * r.k) & 3) * CS];
   }
 }
 
@@ -3601,6 +3657,28 @@ cudaError_t residual(const LevelArgs& L, const ProbArgs& p, const T* u, const T*
         n_vol_chunks, nullptr, sk, sk >= 0 ? p.col_off[sk] : 0, sk >= 0 ? p.col_off[sk + 1] : 0);
     return cudaGetLastError();
   }
+  if (flat_on(L, p) && items && norm && !write_r) {
+    // the stopping test's norm on small and medium levels: one chunk per CTA,
+    // whose partial sums a reduction of up to FLAT_NORM_MAX terms adds up
+    const int* off = sizeof(T) == 8 ? L.gs_off64 : L.gs_off32;
+    const int sk = skip >= 0 && skip < 4 ? skip : -1;
+    const int n_items = sk == 3 ? off[3] : off[4];
+    const int n_if_chunks = (int)lin_grid(n, CTA);
+    const int n_vol_chunks = p.n_act > 0 ? (int)lin_grid((int64_t)n_items * p.n_act, CTA) : 0;
+    const int chunks = n_if_chunks + n_vol_chunks;
+    if (chunks <= FLAT_NORM_MAX) {
+      if (n_part) *n_part = chunks;
+      const bool dep = dep_size(p, chunks) <= DEP_MAX_CTAS;
+      auto kern = seven_point ? (dep ? k_res_flat<T, true, false, true, true> : k_res_flat<T, true, false, true, false>)
+                              : (dep ? k_res_flat<T, false, false, true, true> : k_res_flat<T, false, false, true, false>);
+      ++g_kernel_launches;
+      launch(dep_size(p, chunks), kern, chunks, cta_shape(), 0, s, L.N, L.rs, L.block, u, uI, f, fI, r, W, items,
+             make_int4(off[0], off[1], off[2], off[3]), n_items, p.act, p.n_act, L.cptr, L.cps, L.cp_off, p.free_if, n,
+             if_tab<T>(p, 0), p.zero_off, 0, n_if_chunks, n_vol_chunks, partial, sk, sk >= 0 ? p.col_off[sk] : 0,
+             sk >= 0 ? p.col_off[sk + 1] : 0);
+      return cudaGetLastError();
+    }
+  }
   void (*kern)(int, const int*, int64_t, const T*, const T*, const T*, const T*, T*, const T*, const Tile*, int, const int*,
                int, const int*, const Copy*, const uint32_t*, const int*, int, IfTab<T>, const int64_t*, int, int,
                double*, int*, int, int, int);
@@ -3895,36 +3973,37 @@ cudaError_t fma_probe(double* out, int blocks, int iters, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-cudaError_t reduce_partials(const double* partial, int n, double* out, cudaStream_t s) {
+cudaError_t reduce_partials(const double* partial, int n, double* out, cudaStream_t s, double* host, const int* err,
+                            int* host_err) {
   if (g_rec) return cudaSuccess;   // a batch needs no norms
   ++g_kernel_launches;
-  launch(1, k_reduce, 1, 1024, 0, s, partial, n, out);
+  launch(1, k_reduce, 1, 1024, 0, s, partial, n, out, host, err, host_err);
   return cudaGetLastError();
 }
 
-template <class T>
-cudaError_t import_vec(const LevelArgs& L, const MacroGeo* geo, int n_macro, int64_t nx, int64_t ny, const double* g,
-                       T* blocks, T* masters, bool closed, cudaStream_t s) {
-  (void)masters;
-  // interior imports also go through the closed-lattice tiles (the kernel
-  // filters to the interior)
-  if (L.n_tiles_all > 0) {
-    ++g_kernel_launches;
-    launch((int64_t)L.n_tiles_all * n_macro, k_import_vol<T>, dim3((unsigned)L.n_tiles_all, (unsigned)n_macro), cta_shape(), 0, s,
-        L.N, L.rs, L.block, geo, nx, ny, g, blocks, L.tiles_all, closed);
-  }
+cudaError_t import_problem(const LevelArgs& L, const MacroGeo* geo, int n_macro, int64_t nx, int64_t ny,
+                           const double* gf, const double* gu, double* f, double* fs, const double* winv, double* u,
+                           const int64_t* if_gid, int n_if, double* fI, double* uI, cudaStream_t s) {
+  const int n_if_ctas = (int)lin_grid(n_if, CTA);
+  const int64_t grid = n_if_ctas + (int64_t)L.n_tiles_all * n_macro;
+  if (grid == 0) return cudaSuccess;
+  if (grid > INT32_MAX) return cudaErrorInvalidConfiguration;
+  ++g_kernel_launches;
+  launch(grid, k_import, (unsigned)grid, cta_shape(), 0, s, L.N, L.rs, L.block, geo, nx, ny, gf, gu, f, fs, winv, u,
+         L.tiles_all, L.n_tiles_all, if_gid, n_if, fI, uI, n_if_ctas);
   return cudaGetLastError();
 }
 
-template <class T>
-cudaError_t export_vec(const LevelArgs& L, const MacroGeo* geo, int n_macro, int64_t nx, int64_t ny, const T* blocks,
-                       const T* masters, double* g, cudaStream_t s) {
-  (void)masters;
-  if (L.n_tiles_all > 0) {
-    ++g_kernel_launches;
-    launch((int64_t)L.n_tiles_all * n_macro, k_export_vol<T>, dim3((unsigned)L.n_tiles_all, (unsigned)n_macro), cta_shape(), 0, s,
-        L.N, L.rs, L.block, geo, nx, ny, blocks, g, L.tiles_all);
-  }
+cudaError_t export_solution(const LevelArgs& L, const MacroGeo* geo, int n_macro, int64_t nx, int64_t ny,
+                            const double* u, const double* uI, const int64_t* if_gid, int n_if, double* g,
+                            cudaStream_t s) {
+  const int n_if_ctas = (int)lin_grid(n_if, CTA);
+  const int64_t grid = n_if_ctas + (int64_t)L.n_tiles_all * n_macro;
+  if (grid == 0) return cudaSuccess;
+  if (grid > INT32_MAX) return cudaErrorInvalidConfiguration;
+  ++g_kernel_launches;
+  launch(grid, k_export, (unsigned)grid, cta_shape(), 0, s, L.N, L.rs, L.block, geo, nx, ny, u, uI, g, L.tiles_all,
+         L.n_tiles_all, if_gid, n_if, n_if_ctas);
   return cudaGetLastError();
 }
 
@@ -4156,10 +4235,6 @@ cudaError_t zero_problem_blocks(const LevelArgs& L, const ProbArgs& p, T* u, T* 
                                       cudaStream_t, int, int, int);                                            \
   template cudaError_t coarse_cg<T>(const DevProblem&, const T*, const T*, T*, T*, double, int, cudaStream_t,     \
                                     double*);                                                                  \
-  template cudaError_t import_vec<T>(const LevelArgs&, const MacroGeo*, int, int64_t, int64_t, const double*,    \
-                                     T*, T*, bool, cudaStream_t);                                              \
-  template cudaError_t export_vec<T>(const LevelArgs&, const MacroGeo*, int, int64_t, int64_t, const T*,         \
-                                     const T*, double*, cudaStream_t);                                         \
   template cudaError_t import_masters<T>(const int64_t*, int, const double*, T*, cudaStream_t);                  \
   template cudaError_t export_masters<T>(const int64_t*, int, const T*, double*, cudaStream_t);                  \
   template cudaError_t zero_problem_blocks<T>(const LevelArgs&, const ProbArgs&, T*, T*, cudaStream_t);
