@@ -300,7 +300,9 @@ int hhg_autotune(hhg_mesh* mesh, int reps, int* chosen, void* stream);
  * hhg_batch_launch launches the whole batch with one graph launch on stream;
  * if task_ms is not NULL (n_tasks + 1 doubles, the global task last when
  * present) it synchronises and receives each task's completion time in ms
- * after the start of the launch. */
+ * after the start of the launch.  A batch and its meshes may be destroyed in
+ * either order; the launches and hhg_batch_set_priority return HHG_ERR_STATE
+ * once one of the meshes is gone. */
 typedef struct hhg_batch hhg_batch;
 int hhg_batch_create(hhg_mesh* global, int global_cycles, hhg_mesh* const* meshes, const int* const* ids,
                      const int* n_ids, const int* cycles, int n_tasks, int mixed, hhg_batch** out);

@@ -2035,15 +2035,21 @@ __device__ __forceinline__ double warp_sum_xor(double v) {
 // and the allocation-free cycle) and the cluster form give the same iterates
 // bit for bit.
 //
-// One CTA of CG_THREADS threads: warp w takes the blocks w, w + 8, ... and
-// holds the buckets w, w + 8, w + 16, w + 24 in acc.  buf: 32 doubles;
-// consecutive sums alternate between two buffers.
-__device__ __forceinline__ double cg_allreduce(const double (&acc)[4], double* buf) {
-  const int t = threadIdx.y * blockDim.x + threadIdx.x;   // 1-D or (32, 8) CTAs
-  const int lane = t & 31, w = t >> 5;
-  if (lane < 4) buf[w + CG_WARPS * lane] = lane == 0 ? acc[0] : lane == 1 ? acc[1] : lane == 2 ? acc[2] : acc[3];
-  __syncthreads();
-  return warp_sum_xor(buf[lane]);
+// One CTA of CG_THREADS threads: warp w takes the blocks w, w + 8, ..., four
+// at a time.  Their four trees run as one: after the step over 16 lanes each
+// half of the warp holds two of them, after the step over 8 each quarter one,
+// so four blocks cost six additions instead of twenty (one CTA is bound by the
+// FP64 pipe: with a tree per block the persistent batch with a 3375-row coarse
+// problem took 248 ms instead of 210).  Quarter e of the warp ends with block
+// e's sum, the same bits as warp_sum_xor, and holds bucket w + 8 e.
+__device__ __forceinline__ double warp_sum4(const double (&v)[4]) {
+  const bool h16 = (threadIdx.x & 16) != 0, h8 = (threadIdx.x & 8) != 0;
+  const double a = __dadd_rn(h16 ? v[2] : v[0], __shfl_xor_sync(0xffffffffu, h16 ? v[0] : v[2], 16));
+  const double b = __dadd_rn(h16 ? v[3] : v[1], __shfl_xor_sync(0xffffffffu, h16 ? v[1] : v[3], 16));
+  double s = __dadd_rn(h8 ? b : a, __shfl_xor_sync(0xffffffffu, h8 ? a : b, 8));
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) s = __dadd_rn(s, __shfl_xor_sync(0xffffffffu, s, o));
+  return s;
 }
 
 // Rows per lane of a block (as a shift): from 16385 rows on a block has 128
@@ -2052,29 +2058,31 @@ __device__ __forceinline__ double cg_allreduce(const double (&acc)[4], double* b
 __host__ __device__ __forceinline__ int cg_block_shift(int n) { return n > 16384 ? 2 : 0; }
 
 // Calls body(q) -> double for the rows q of the warp's blocks and returns the
-// sum over all rows (to every thread).
+// sum over all rows (to every thread).  buf: 32 doubles; consecutive sums
+// alternate between two buffers.
 template <class F>
 __device__ __forceinline__ double cg_rows_sum(int n, double* buf, F&& body) {
-  const int t = threadIdx.y * blockDim.x + threadIdx.x;
+  const int t = threadIdx.y * blockDim.x + threadIdx.x;   // 1-D or (32, 8) CTAs
   const int lane = t & 31, w = t >> 5;
   const int sh = cg_block_shift(n);
   const int nb = ((n - 1) >> (5 + sh)) + 1;
-  double acc[4] = {0.0, 0.0, 0.0, 0.0};
+  double acc = 0.0;
   for (int b0 = w; b0 < nb; b0 += 32) {
+    double v[4];
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
       const int b = b0 + CG_WARPS * e;
-      if (b < nb) {
-        double v = 0.0;
-        for (int g = 0; g < 1 << sh; ++g) {
-          const int q = ((b << sh) + g) * 32 + lane;
-          if (q < n) v = g ? __dadd_rn(v, body(q)) : body(q);
-        }
-        acc[e] += warp_sum_xor(v);
+      v[e] = 0.0;
+      for (int g = 0; b < nb && g < 1 << sh; ++g) {
+        const int q = ((b << sh) + g) * 32 + lane;
+        if (q < n) v[e] = g ? __dadd_rn(v[e], body(q)) : body(q);
       }
     }
+    acc += warp_sum4(v);
   }
-  return cg_allreduce(acc, buf);
+  if ((lane & 7) == 0) buf[w + CG_WARPS * (lane >> 3)] = acc;
+  __syncthreads();
+  return warp_sum_xor(buf[lane]);
 }
 
 // 1 / b, about one unit in the last place: the hardware's reciprocal
@@ -2140,12 +2148,21 @@ __device__ __forceinline__ void cg_one_cta(int n, const int* rowptr, const int* 
                                            int* iters, double* red) {
   const int t = threadIdx.y * blockDim.x + threadIdx.x;
   auto z = [&](int q) { return dinv ? dinv[q] * r[q] : r[q]; };
-  auto row_times = [&](int q) {
+  auto row_times = [&](int q) {   // entries four at a time, their loads together
     double a0 = 0.0, a1 = 0.0;
-    const int e1 = rowptr[q + 1];
-    for (int e = rowptr[q]; e < e1; e += 2) {
-      a0 = fma(val[e], z(col[e]), a0);
-      if (e + 1 < e1) a1 = fma(val[e + 1], z(col[e + 1]), a1);
+    const int e0 = rowptr[q], e1 = rowptr[q + 1];
+    for (int e = e0; e < e1; e += 4) {
+      double zv[4], wv[4];
+#pragma unroll
+      for (int x = 0; x < 4; ++x) {
+        const int at = e + x < e1 ? e + x : e;
+        wv[x] = val[at];
+        zv[x] = z(col[at]);
+      }
+      a0 = fma(wv[0], zv[0], a0);
+      if (e + 1 < e1) a1 = fma(wv[1], zv[1], a1);
+      if (e + 2 < e1) a0 = fma(wv[2], zv[2], a0);
+      if (e + 3 < e1) a1 = fma(wv[3], zv[3], a1);
     }
     return a0 + a1;
   };
@@ -2153,7 +2170,7 @@ __device__ __forceinline__ void cg_one_cta(int n, const int* rowptr, const int* 
   double rz = cg_rows_sum(n, red, [&](int q) {
     const int64_t src = fsrc[q];
     const double b = src >= 0 ? (double)f[src] : (double)fI[-1 - src];
-    x[q] = 0.0;
+    x[q] = p[q] = s[q] = 0.0;
     r[q] = b;
     return b * z(q);
   });
@@ -2165,9 +2182,10 @@ __device__ __forceinline__ void cg_one_cta(int n, const int* rowptr, const int* 
   while (bnorm > 0.0 && it < maxit && cg_above(rr, test)) {
     __syncthreads();   // every r entry is written, every total read
     const double pAp = cg_rows_sum(n, red + 32, [&](int q) {
+      const double p0 = p[q], s0 = s[q], zq = z(q);   // zero in the first iteration, as beta
       const double w = row_times(q);
-      const double pq = it ? fma(beta, p[q], z(q)) : z(q);
-      const double sq = it ? fma(beta, s[q], w) : w;
+      const double pq = fma(beta, p0, zq);
+      const double sq = fma(beta, s0, w);
       p[q] = pq;
       s[q] = sq;
       return pq * sq;
@@ -3175,7 +3193,7 @@ _Pragma("unroll")
 
 // Coarse CG (k_cg with its vectors in the problem's global work array).
 template <class T>
-__device__ void unit_cg(const BOp& op, double* red) {
+__device__ __noinline__ void unit_cg(const BOp& op, double* red) {
   const size_t n = (size_t)op.n_cg;
   cg_one_cta<T>(op.n_cg, op.rowptr, op.col, op.val, op.fsrc, (const T*)op.f, (const T*)op.fI, op.uptr, op.udst,
                 op.umaster, (T*)op.u, (T*)op.uI, op.work, op.work + n, op.work + 2 * n, op.work + 3 * n, op.dinv,
