@@ -59,6 +59,15 @@ constexpr int CTA = TILE_ROWS * TILE_SLOTS;   // 256 threads, 32 x 8
 // it a kernel touches only tables written at set-up (work items, active macros,
 // lists, copy pointers, stencil weights), which host-synchronous copies wrote.
 // Every kernel calls it, so completion stays in stream order.
+//
+// The vectors (iterates, loads, residuals, partial sums) may change while such
+// a kernel is resident and waits.  So its vector parameters are not
+// __restrict__ (the compiler could move their loads above the wait, or send
+// them through the read-only path, which is defined for data that stays the
+// same as long as the kernel lives), and they are read with plain loads: the
+// read-only path is left to launches that do not overlap (NC = !DEP below).
+// The functions called after the wait may declare theirs __restrict__ again,
+// which says nothing about the time before the call.
 __device__ __forceinline__ void launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void after_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
@@ -458,7 +467,8 @@ struct Vec;
 // load<true>() goes through the read-only path: a Gauss-Seidel colour
 // kernel reads only arrays it does not write (the other colours and f).
 // load<false>() is a plain coherent load, for code that reads data written
-// earlier in the same launch (the persistent batch executor).
+// earlier in the same launch (the persistent batch executor) or while the
+// launch waited for its predecessor (DEP kernels).
 template <>
 struct Vec<float> {
   static constexpr int n = 4;
@@ -747,18 +757,18 @@ __device__ __forceinline__ void gs_tile7(const Tile& t, int N, const int* __rest
 
 // fs / Wsc (7-point only, may be null): the volume nodes read f and the
 // interior weights already divided by their macro's centre weight.
-template <class T, bool S7>
-__global__ void __launch_bounds__(CTA, 5) k_gs(int N, const int* __restrict__ rs, int64_t block, T* __restrict__ u, T* __restrict__ uI,
-                                            const T* __restrict__ f, const T* __restrict__ fI,
+template <class T, bool S7, bool DEP>
+__global__ void __launch_bounds__(CTA, 5) k_gs(int N, const int* __restrict__ rs, int64_t block, T* u, T* uI,
+                                            const T* f, const T* fI,
                                             const T* __restrict__ W, const T* __restrict__ Winv,
-                                            const T* __restrict__ fs, const T* __restrict__ Wsc,
+                                            const T* fs, const T* __restrict__ Wsc,
                                             const Tile* __restrict__ tiles, int n_tiles, const int* __restrict__ act,
                                             int n_act, int colour, const int* __restrict__ cptr,
                                             const Copy* __restrict__ cps, const uint32_t* __restrict__ cpo,
                                             const int* __restrict__ list, int n_list, IfTab<T> tab,
-                                            int n_if_units, int* __restrict__ sched) {
-  launch_next();
-  after_previous();
+                                            int n_if_units, int* sched) {
+  if (DEP) launch_next();
+  if (DEP) after_previous();
   __shared__ int s_pre2[MAX_SLABS][33];
   __shared__ int s_pre_tot[MAX_SLABS + 1];
   __shared__ int s_unit;
@@ -791,10 +801,10 @@ __global__ void __launch_bounds__(CTA, 5) k_gs(int N, const int* __restrict__ rs
     const T inv = Winv[macro];
     if (S7) {
       if (Wsc)
-        gs_tile7<T, true>(t, N, rs, colour, ub, fs + (size_t)macro * block, Wsc + (size_t)macro * 16 * NDIR, T(1),
-                          s_pre2, s_pre_tot);
+        gs_tile7<T, true, !DEP>(t, N, rs, colour, ub, fs + (size_t)macro * block, Wsc + (size_t)macro * 16 * NDIR,
+                                T(1), s_pre2, s_pre_tot);
       else
-        gs_tile7<T, false>(t, N, rs, colour, ub, fb, w, inv, s_pre2, s_pre_tot);
+        gs_tile7<T, false, !DEP>(t, N, rs, colour, ub, fb, w, inv, s_pre2, s_pre_tot);
     } else {
       // 15-point: one colour-c node per item
       const int total = flat_setup_slabs(t, N, colour, true, 1, s_pre2, s_pre_tot);
@@ -852,8 +862,8 @@ struct FlatMinCtas {
 // sum in the same order as if_offdiag.
 template <class T, bool S7>
 __device__ __forceinline__ void gs_if_prefetched(const IfTab<T>& tab, int q, int node, int c0, int c1,
-                                                 const uint32_t* __restrict__ cpo, T* __restrict__ u,
-                                                 T* __restrict__ uI, const T* __restrict__ fI) {
+                                                 const uint32_t* __restrict__ cpo, T* u,
+                                                 T* uI, const T* fI) {
   constexpr int PRE = S7 ? 6 : 16;
   const bool var = !S7 && tab.ptr;
   const int n = var ? tab.len[q] : if_tab_k(S7);
@@ -891,10 +901,10 @@ __device__ __forceinline__ void gs_if_prefetched(const IfTab<T>& tab, int q, int
 }
 
 template <class T, bool S7, bool SCALED, bool DEP>
-__global__ void __launch_bounds__(CTA, S7 && !DEP ? FlatMinCtas<T>::value : 0) k_gs_flat(int N, const int* __restrict__ rs, int64_t block, T* __restrict__ u,
-                                                 T* __restrict__ uI, const T* __restrict__ fI,
+__global__ void __launch_bounds__(CTA, S7 && !DEP ? FlatMinCtas<T>::value : 0) k_gs_flat(int N, const int* __restrict__ rs, int64_t block, T* u,
+                                                 T* uI, const T* fI,
                                                  const T* __restrict__ W, const T* __restrict__ Winv,
-                                                 const T* __restrict__ fv, const T* __restrict__ Wv,
+                                                 const T* fv, const T* __restrict__ Wv,
                                                  const uint32_t* __restrict__ items, int n_items,
                                                  const int* __restrict__ act, int n_act, int colour,
                                                  const int* __restrict__ cptr, const Copy* __restrict__ cps,
@@ -941,15 +951,15 @@ __global__ void __launch_bounds__(CTA, S7 && !DEP ? FlatMinCtas<T>::value : 0) k
       const Slice sc = slice_consts(rs, N, k);
       const T inv = SCALED ? T(1) : Winv[macro];
       after_previous();
-      gs_group7<T, SCALED>(sc, N, j, g, colour, u + (size_t)macro * block, fv + (size_t)macro * block, wr, inv);
+      gs_group7<T, SCALED, !DEP>(sc, N, j, g, colour, u + (size_t)macro * block, fv + (size_t)macro * block, wr, inv);
     } else {
-      gs_group7<T, SCALED>(slice_consts(rs, N, k), N, j, g, colour, u + (size_t)macro * block,
+      gs_group7<T, SCALED, !DEP>(slice_consts(rs, N, k), N, j, g, colour, u + (size_t)macro * block,
                            fv + (size_t)macro * block, wr, SCALED ? T(1) : Winv[macro]);
     }
   } else {
     const Slice sc = slice_consts(rs, N, k);
     if (DEP) after_previous();
-    gs_group15<T>(sc, N, j, g, colour, u + (size_t)macro * block, fv + (size_t)macro * block, w, Winv[macro]);
+    gs_group15<T, !DEP>(sc, N, j, g, colour, u + (size_t)macro * block, fv + (size_t)macro * block, w, Winv[macro]);
   }
 }
 
@@ -1114,12 +1124,12 @@ constexpr int STREAM_CTA = 32 * (STREAM_CONSUMERS + 1);
 
 template <class T, bool SCALED>
 __global__ void __launch_bounds__(STREAM_CTA) k_gs_stream(
-    int N, const int* __restrict__ rs, int64_t block, T* __restrict__ u, T* __restrict__ uI,
-    const T* __restrict__ fI, const T* __restrict__ W, const T* __restrict__ Winv, const T* __restrict__ fv,
+    int N, const int* __restrict__ rs, int64_t block, T* u, T* uI,
+    const T* fI, const T* __restrict__ W, const T* __restrict__ Winv, const T* fv,
     const T* __restrict__ Wv, const StreamTile* __restrict__ tiles, int n_tiles, const int* __restrict__ act,
     int n_act, int colour, const int* __restrict__ cptr, const Copy* __restrict__ cps,
     const uint32_t* __restrict__ cpo, const int* __restrict__ list, int n_list, IfTab<T> tab, int n_if_units,
-    int* __restrict__ sched, int slot, int wait_limit, int* __restrict__ err) {
+    int* sched, int slot, int wait_limit, int* err) {
   launch_next();
   after_previous();
   extern __shared__ __align__(128) unsigned char s_dyn[];
@@ -1299,19 +1309,42 @@ __global__ void __launch_bounds__(STREAM_CTA) k_gs_stream(
 // Residual r = f - A u on the free nodes (all colours); optional write of r
 // (zero at the problem's frozen ghost copies) and per-CTA partial sums of r^2
 // ---------------------------------------------------------------------------
-template <class T, bool S7, bool WRITE, bool NORM>
-__global__ void __launch_bounds__(CTA, 4) k_res(int N, const int* __restrict__ rs, int64_t block, const T* __restrict__ u,
-                                             const T* __restrict__ uI, const T* __restrict__ f,
-                                             const T* __restrict__ fI, T* __restrict__ r, const T* __restrict__ W,
+// The 15-point items of one tile: four nodes of one slot each.
+template <class T, bool WRITE, bool NORM>
+__device__ __forceinline__ void res_tile15(const Tile& t, int N, const int* __restrict__ rs,
+                                           const T* __restrict__ ub, const T* __restrict__ fb, T* __restrict__ rb,
+                                           const T* __restrict__ w, int skip, double& ss, int (*s_pre2)[33],
+                                           int* s_pre_tot) {
+  HHG_TILE_NODES(N, rs, t, s_pre, {
+    const int me = lidx32(rs, N, i, j, k);
+    T acc = T(0);
+    if (((i + 2 * j + 3 * k) & 3) != skip) {
+      acc = fb[me] - w[0] * ub[me];
+_Pragma("unroll")
+      for (int d = 1; d < NDIR; ++d) {
+        int di, dj, dk;
+        dir_ijk(d, di, dj, dk);
+        acc -= w[d] * ub[lidx32(rs, N, i + di, j + dj, k + dk)];
+      }
+    }
+    if (WRITE) rb[me] = acc;
+    if (NORM) ss += (double)acc * (double)acc;
+  })
+}
+
+template <class T, bool S7, bool WRITE, bool NORM, bool DEP>
+__global__ void __launch_bounds__(CTA, 4) k_res(int N, const int* __restrict__ rs, int64_t block, const T* u,
+                                             const T* uI, const T* f,
+                                             const T* fI, T* r, const T* __restrict__ W,
                                              const Tile* __restrict__ tiles, int n_tiles, const int* __restrict__ act,
                                              int n_act, const int* __restrict__ cptr, const Copy* __restrict__ cps,
                                              const uint32_t* __restrict__ cpo, const int* __restrict__ list,
                                              int n_list, IfTab<T> tab,
                                              const int64_t* __restrict__ zero_off, int n_zero, int n_if_units,
-                                             double* __restrict__ partial, int* __restrict__ sched, int skip,
+                                             double* partial, int* sched, int skip,
                                              int skip_lo, int skip_hi) {
-  launch_next();
-  after_previous();
+  if (DEP) launch_next();
+  if (DEP) after_previous();
   __shared__ int s_pre2[MAX_SLABS][33];
   __shared__ int s_pre_tot[MAX_SLABS + 1];
   __shared__ double sh[32];
@@ -1365,28 +1398,13 @@ __global__ void __launch_bounds__(CTA, 4) k_res(int N, const int* __restrict__ r
           if (c == skip)
             res_group7<T, WRITE, NORM, true>(slice_consts(rs, N, k), N, j, g, c, ub, fb, rb, wr, ss);
           else
-            res_group7<T, WRITE, NORM>(slice_consts(rs, N, k), N, j, g, c, ub, fb, rb, wr, ss);
+            res_group7<T, WRITE, NORM, false, !DEP>(slice_consts(rs, N, k), N, j, g, c, ub, fb, rb, wr, ss);
         }
         __syncthreads();
       }
       continue;
     }
-    // 15-point: four nodes of one slot per item
-    HHG_TILE_NODES(N, rs, t, s_pre, {
-      const int me = lidx32(rs, N, i, j, k);
-      T acc = T(0);
-      if (((i + 2 * j + 3 * k) & 3) != skip) {
-        acc = fb[me] - w[0] * ub[me];
-_Pragma("unroll")
-        for (int d = 1; d < NDIR; ++d) {
-          int di, dj, dk;
-          dir_ijk(d, di, dj, dk);
-          acc -= w[d] * ub[lidx32(rs, N, i + di, j + dj, k + dk)];
-        }
-      }
-      if (WRITE) rb[me] = acc;
-      if (NORM) ss += (double)acc * (double)acc;
-    })
+    res_tile15<T, WRITE, NORM>(t, N, rs, ub, fb, rb, w, skip, ss, s_pre2, s_pre_tot);
   }
   finish_units(sched, n_if_units + n_tiles * n_act);
   if (NORM) {
@@ -1406,15 +1424,15 @@ _Pragma("unroll")
 // colour 3).
 template <class T, bool S7, bool WRITE, bool NORM, bool DEP>
 __global__ void __launch_bounds__(CTA) k_res_flat(int N, const int* __restrict__ rs, int64_t block,
-                                                  const T* __restrict__ u, const T* __restrict__ uI,
-                                                  const T* __restrict__ f, const T* __restrict__ fI, T* __restrict__ r,
+                                                  const T* u, const T* uI,
+                                                  const T* f, const T* fI, T* r,
                                                   const T* __restrict__ W, const uint32_t* __restrict__ items,
                                                   int4 off, int n_items, const int* __restrict__ act, int n_act,
                                                   const int* __restrict__ cptr, const Copy* __restrict__ cps,
                                                   const uint32_t* __restrict__ cpo, const int* __restrict__ list,
                                                   int n_list, IfTab<T> tab, const int64_t* __restrict__ zero_off,
                                                   int n_zero, int n_if_chunks, int n_vol_chunks,
-                                                  double* __restrict__ partial, int skip, int skip_lo, int skip_hi) {
+                                                  double* partial, int skip, int skip_lo, int skip_hi) {
   __shared__ double sh[32];
   double ss = 0.0;
   const int n_vol = n_items * n_act;
@@ -1459,10 +1477,10 @@ __global__ void __launch_bounds__(CTA) k_res_flat(int N, const int* __restrict__
     if constexpr (S7) {
       const T wr[11] = {w[0], w[1], w[2], w[3], T(0), T(0), T(0), T(0), w[8], w[9], w[10]};
       if (c == skip) res_group7<T, WRITE, NORM, true>(sc, N, j, g, c, u + mb, f + mb, r + mb, wr, ss);
-      else res_group7<T, WRITE, NORM>(sc, N, j, g, c, u + mb, f + mb, r + mb, wr, ss);
+      else res_group7<T, WRITE, NORM, false, !DEP>(sc, N, j, g, c, u + mb, f + mb, r + mb, wr, ss);
     } else {
       if (c == skip) res_group15<T, WRITE, NORM, true>(sc, N, j, g, c, u + mb, f + mb, r + mb, w, ss);
-      else res_group15<T, WRITE, NORM>(sc, N, j, g, c, u + mb, f + mb, r + mb, w, ss);
+      else res_group15<T, WRITE, NORM, false, !DEP>(sc, N, j, g, c, u + mb, f + mb, r + mb, w, ss);
     }
   }
   if (NORM) {
@@ -1551,18 +1569,18 @@ __device__ __forceinline__ void restrict_tile(const Tile& t, int Nc, const int* 
   });
 }
 
-template <class T>
-__global__ void __launch_bounds__(CTA, 4) k_restrict(int Nc, const int* __restrict__ rsc, int64_t bc, T* __restrict__ fc, T* __restrict__ fIc,
-                                                  T* __restrict__ uc, T* __restrict__ uIc, int Nf, const int* __restrict__ rsf, int64_t bf,
-                                                  const T* __restrict__ rf, const Tile* __restrict__ tiles, int n_tiles,
+template <class T, bool DEP>
+__global__ void __launch_bounds__(CTA, 4) k_restrict(int Nc, const int* __restrict__ rsc, int64_t bc, T* fc, T* fIc,
+                                                  T* uc, T* uIc, int Nf, const int* __restrict__ rsf, int64_t bf,
+                                                  const T* rf, const Tile* __restrict__ tiles, int n_tiles,
                                                   const int* __restrict__ act, int n_act,
                                                   const int* __restrict__ cptr, const Copy* __restrict__ cps,
                                                   const uint32_t* __restrict__ cpo,
                                                   const int* __restrict__ list, int n_list,
                                                   const int64_t* __restrict__ gather,
-                                                  const int64_t* __restrict__ zero_off, int n_zero, int n_if_units, int* __restrict__ sched) {
-  launch_next();
-  after_previous();
+                                                  const int64_t* __restrict__ zero_off, int n_zero, int n_if_units, int* sched) {
+  if (DEP) launch_next();
+  if (DEP) after_previous();
   __shared__ int s_pre2[MAX_SLABS][33];
   __shared__ int s_pre_tot[MAX_SLABS + 1];
   __shared__ int s_unit;
@@ -1588,7 +1606,7 @@ __global__ void __launch_bounds__(CTA, 4) k_restrict(int Nc, const int* __restri
     Tile t;
     int macro;
     vol_subunit(vol_index(unit, n_if_units), n_act, RESTRICT_SPLIT, tiles, act, t, macro);
-    restrict_tile<T, true>(t, Nc, rsc, Nf, rsf, rf + (size_t)macro * bf, fc + (size_t)macro * bc,
+    restrict_tile<T, !DEP>(t, Nc, rsc, Nf, rsf, rf + (size_t)macro * bf, fc + (size_t)macro * bc,
                            uc + (size_t)macro * bc, s_pre2, s_pre_tot);
   }
   finish_units(sched, n_if_units + n_tiles * RESTRICT_SPLIT * n_act);
@@ -1755,17 +1773,17 @@ __device__ __forceinline__ void prolong_tile(const Tile& t, int Nf, const int* _
   }
 }
 
-template <class T>
-__global__ void __launch_bounds__(CTA) k_prolong(int Nf, const int* __restrict__ rsf, int64_t bf, T* __restrict__ uf, T* __restrict__ uIf,
-                                                 int Nc, const int* __restrict__ rsc, int64_t bc, const T* __restrict__ uc,
+template <class T, bool DEP>
+__global__ void __launch_bounds__(CTA) k_prolong(int Nf, const int* __restrict__ rsf, int64_t bf, T* uf, T* uIf,
+                                                 int Nc, const int* __restrict__ rsc, int64_t bc, const T* uc,
                                                  const Tile* __restrict__ tiles, int n_tiles,
                                                  const int* __restrict__ act, int n_act, const int* __restrict__ cptr,
                                                  const Copy* __restrict__ cps, const uint32_t* __restrict__ cpo,
                                                  const int* __restrict__ list,
-                                                 int n_list, int n_if_units, int* __restrict__ sched, int skip,
+                                                 int n_list, int n_if_units, int* sched, int skip,
                                                  int if_lo, int if_hi) {
-  launch_next();
-  after_previous();
+  if (DEP) launch_next();
+  if (DEP) after_previous();
   __shared__ int s_pre2[MAX_SLABS][33];
   __shared__ int s_pre_tot[MAX_SLABS + 1];
   __shared__ int s_unit;
@@ -1785,7 +1803,7 @@ __global__ void __launch_bounds__(CTA) k_prolong(int Nf, const int* __restrict__
     Tile t;
     int macro;
     vol_unit(vol_index(unit, n_if_units), n_act, tiles, act, t, macro);
-    prolong_tile<T, true>(t, Nf, rsf, Nc, rsc, uf + (size_t)macro * bf, uc + (size_t)macro * bc, skip, s_pre2,
+    prolong_tile<T, !DEP>(t, Nf, rsf, Nc, rsc, uf + (size_t)macro * bf, uc + (size_t)macro * bc, skip, s_pre2,
                           s_pre_tot);
   }
   finish_units(sched, n_if_units + n_tiles * n_act);
@@ -1800,9 +1818,9 @@ __global__ void __launch_bounds__(CTA) k_prolong(int Nf, const int* __restrict__
 // node as k_restrict / k_prolong, so the same values bit for bit.
 template <class T, bool DEP>
 __global__ void __launch_bounds__(CTA) k_restrict_flat(int Nc, const int* __restrict__ rsc, int64_t bc,
-                                                       T* __restrict__ fc, T* __restrict__ fIc, T* __restrict__ uc,
-                                                       T* __restrict__ uIc, int Nf, const int* __restrict__ rsf,
-                                                       int64_t bf, const T* __restrict__ rf,
+                                                       T* fc, T* fIc, T* uc,
+                                                       T* uIc, int Nf, const int* __restrict__ rsf,
+                                                       int64_t bf, const T* rf,
                                                        const uint32_t* __restrict__ slots, int n_slots,
                                                        const int* __restrict__ act, int n_act,
                                                        const int* __restrict__ cptr, const Copy* __restrict__ cps,
@@ -1838,7 +1856,7 @@ __global__ void __launch_bounds__(CTA) k_restrict_flat(int Nc, const int* __rest
   const int macro = act[a];
   const uint32_t d = slots[it];
   if (DEP) after_previous();
-  restrict_slot<T, true>(Nc, rsc, Nf, rsf, (int)(d >> 20), (int)((d >> 10) & 1023u), (int)(d & 1023u),
+  restrict_slot<T, !DEP>(Nc, rsc, Nf, rsf, (int)(d >> 20), (int)((d >> 10) & 1023u), (int)(d & 1023u),
                          rf + (size_t)macro * bf, fc + (size_t)macro * bc, uc + (size_t)macro * bc);
 }
 
@@ -1848,9 +1866,9 @@ __global__ void __launch_bounds__(CTA) k_restrict_flat(int Nc, const int* __rest
 // colour.
 template <class T, bool DEP>
 __global__ void __launch_bounds__(CTA) k_prolong_flat(int Nf, const int* __restrict__ rsf, int64_t bf,
-                                                      T* __restrict__ uf, T* __restrict__ uIf, int Nc,
+                                                      T* uf, T* uIf, int Nc,
                                                       const int* __restrict__ rsc, int64_t bc,
-                                                      const T* __restrict__ uc, const uint32_t* __restrict__ items,
+                                                      const T* uc, const uint32_t* __restrict__ items,
                                                       int n_items, int first_c, int3 off,
                                                       const int* __restrict__ act, int n_act,
                                                       const int* __restrict__ cptr, const Copy* __restrict__ cps,
@@ -1880,7 +1898,7 @@ __global__ void __launch_bounds__(CTA) k_prolong_flat(int Nf, const int* __restr
   const int macro = act[a];
   const uint32_t d = items[it];
   if (DEP) after_previous();
-  prolong_group<T, true>(Nf, rsf, Nc, rsc, (int)(d >> 20), (int)((d >> 10) & 1023u), (int)(d & 1023u), c,
+  prolong_group<T, !DEP>(Nf, rsf, Nc, rsc, (int)(d >> 20), (int)((d >> 10) & 1023u), (int)(d & 1023u), c,
                          uf + (size_t)macro * bf, uc + (size_t)macro * bc);
 }
 
@@ -1889,16 +1907,49 @@ __global__ void __launch_bounds__(CTA) k_prolong_flat(int Nf, const int* __restr
 // side (with partial sums of r^2), and the FP64 update u += e
 // ---------------------------------------------------------------------------
 template <bool S7>
-__global__ void __launch_bounds__(CTA) k_res_f32(int N, const int* __restrict__ rs, int64_t block, const double* __restrict__ u,
-                                                 const double* __restrict__ uI, const double* __restrict__ f,
-                                                 const double* __restrict__ fI, float* __restrict__ f32,
-                                                 float* __restrict__ fI32, const double* __restrict__ W,
+__device__ __forceinline__ void res_f32_tile(const Tile& t, int N, const int* __restrict__ rs,
+                                             const double* __restrict__ ub, const double* __restrict__ fb,
+                                             float* __restrict__ ob, const double* __restrict__ w, double& ss,
+                                             int (*s_pre2)[33], int* s_pre_tot) {
+  HHG_TILE_NODES(N, rs, t, s_pre, {
+    int me;
+    double acc;
+    if (S7) {
+      const Nb7 q = nb7(sc, i, j);
+      me = q.me;
+      acc = fb[me] - w[0] * ub[me];
+      acc -= w[1] * ub[q.nb1];
+      acc -= w[2] * ub[q.nb2];
+      acc -= w[3] * ub[q.nb3];
+      acc -= w[8] * ub[q.nb8];
+      acc -= w[9] * ub[q.nb9];
+      acc -= w[10] * ub[q.nb10];
+    } else {
+      me = lidx32(rs, N, i, j, k);
+      acc = fb[me] - w[0] * ub[me];
+_Pragma("unroll")
+      for (int d = 1; d < NDIR; ++d) {
+        int di, dj, dk;
+        dir_ijk(d, di, dj, dk);
+        acc -= w[d] * ub[lidx32(rs, N, i + di, j + dj, k + dk)];
+      }
+    }
+    ob[me] = (float)acc;
+    ss += acc * acc;
+  })
+}
+
+template <bool S7>
+__global__ void __launch_bounds__(CTA) k_res_f32(int N, const int* __restrict__ rs, int64_t block, const double* u,
+                                                 const double* uI, const double* f,
+                                                 const double* fI, float* f32,
+                                                 float* fI32, const double* __restrict__ W,
                                                  const Tile* __restrict__ tiles, int n_tiles,
                                                  const int* __restrict__ act, int n_act,
                                                  const int* __restrict__ cptr, const Copy* __restrict__ cps,
                                                  const int* __restrict__ list, int n_list, IfTab<double> tab,
-                                                 int n_if_units, double* __restrict__ partial,
-                                                 int* __restrict__ sched) {
+                                                 int n_if_units, double* partial,
+                                                 int* sched) {
   launch_next();
   after_previous();
   __shared__ int s_pre2[MAX_SLABS][33];
@@ -1932,32 +1983,7 @@ __global__ void __launch_bounds__(CTA) k_res_f32(int N, const int* __restrict__ 
     const double* fb = f + (size_t)macro * block;
     float* ob = f32 + (size_t)macro * block;
     const double* w = W + (size_t)macro * 16 * NDIR;
-    HHG_TILE_NODES(N, rs, t, s_pre, {
-      int me;
-      double acc;
-      if (S7) {
-        const Nb7 q = nb7(sc, i, j);
-        me = q.me;
-        acc = fb[me] - w[0] * ub[me];
-        acc -= w[1] * ub[q.nb1];
-        acc -= w[2] * ub[q.nb2];
-        acc -= w[3] * ub[q.nb3];
-        acc -= w[8] * ub[q.nb8];
-        acc -= w[9] * ub[q.nb9];
-        acc -= w[10] * ub[q.nb10];
-      } else {
-        me = lidx32(rs, N, i, j, k);
-        acc = fb[me] - w[0] * ub[me];
-_Pragma("unroll")
-        for (int d = 1; d < NDIR; ++d) {
-          int di, dj, dk;
-          dir_ijk(d, di, dj, dk);
-          acc -= w[d] * ub[lidx32(rs, N, i + di, j + dj, k + dk)];
-        }
-      }
-      ob[me] = (float)acc;
-      ss += acc * acc;
-    })
+    res_f32_tile<S7>(t, N, rs, ub, fb, ob, w, ss, s_pre2, s_pre_tot);
   }
   finish_units(sched, n_if_units + n_tiles * n_act);
   const double s = block_sum(ss, sh);
@@ -1969,24 +1995,25 @@ _Pragma("unroll")
 // frozen copies, padding; the blocks are cleared before the cycle), and each
 // ghost copy of a free interface node holds the master's correction, so the
 // copies stay equal to their masters.  Blocks are multiples of 256 slots.
-__global__ void __launch_bounds__(256) k_add_corr_blocks(double* __restrict__ u, const float* __restrict__ e,
-                                                        int64_t block, const int* __restrict__ act) {
-  launch_next();
-  after_previous();
-  const size_t base = (size_t)act[blockIdx.y] * block;
-  double2* ub = reinterpret_cast<double2*>(u + base);
-  const float2* eb = reinterpret_cast<const float2*>(e + base);
-  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < block / 2; q += (int64_t)gridDim.x * blockDim.x) {
+__device__ __forceinline__ void add_corr(double2* __restrict__ ub, const float2* __restrict__ eb, int64_t n) {
+  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += (int64_t)gridDim.x * blockDim.x) {
     double2 x = ub[q];
-    const float2 d = __ldg(eb + q);
+    const float2 d = eb[q];
     x.x += (double)d.x;
     x.y += (double)d.y;
     ub[q] = x;
   }
 }
+__global__ void __launch_bounds__(256) k_add_corr_blocks(double* u, const float* e, int64_t block,
+                                                        const int* __restrict__ act) {
+  launch_next();
+  after_previous();
+  const size_t base = (size_t)act[blockIdx.y] * block;
+  add_corr(reinterpret_cast<double2*>(u + base), reinterpret_cast<const float2*>(e + base), block / 2);
+}
 
 // uI[list[q]] += eI[list[q]] for the free interface masters.
-__global__ void k_add_corr_masters(double* __restrict__ uI, const float* __restrict__ eI, const int* __restrict__ list,
+__global__ void k_add_corr_masters(double* uI, const float* eI, const int* __restrict__ list,
                                    int n) {
   launch_next();
   after_previous();
@@ -2217,12 +2244,12 @@ __device__ __forceinline__ void cg_one_cta(int n, const int* rowptr, const int* 
 template <class T>
 __global__ void __launch_bounds__(CG_THREADS) k_cg(int n, const int* __restrict__ rowptr, const int* __restrict__ col,
                                                    const double* __restrict__ val, const int64_t* __restrict__ fsrc,
-                                                   const T* __restrict__ f, const T* __restrict__ fI,
+                                                   const T* f, const T* fI,
                                                    const int* __restrict__ uptr, const int64_t* __restrict__ udst,
-                                                   const int* __restrict__ umaster, T* __restrict__ u,
-                                                   T* __restrict__ uI, double* __restrict__ work,
+                                                   const int* __restrict__ umaster, T* u,
+                                                   T* uI, double* work,
                                                    const double* __restrict__ dinv, double rtol, int maxit,
-                                                   int* __restrict__ iters) {
+                                                   int* iters) {
   launch_next();
   after_previous();
   __shared__ double red[64];
@@ -2305,9 +2332,9 @@ __device__ __forceinline__ double cg_total(const double* sums, int nb) {
 // row in shared memory.  NB = 0 (large coarse problems): any number of blocks,
 // x, p, s and A r in the work array and the matrix read from its CSR arrays.
 template <class T, int NB, int KC, bool JAC>
-__global__ void __launch_bounds__(NB > 0 ? CG_THREADS + 32 : 1024) k_cg_cluster(CgArgs A, const T* __restrict__ f,
-                                                                const T* __restrict__ fI, T* __restrict__ u,
-                                                                T* __restrict__ uI) {
+__global__ void __launch_bounds__(NB > 0 ? CG_THREADS + 32 : 1024) k_cg_cluster(CgArgs A, const T* f,
+                                                                const T* fI, T* u,
+                                                                T* uI) {
   launch_next();
   extern __shared__ double s_cg[];
   __shared__ double s_alpha, s_beta;
@@ -2530,9 +2557,9 @@ __global__ void __launch_bounds__(NB > 0 ? CG_THREADS + 32 : 1024) k_cg_cluster(
 // macro's own sub-stencil at p applied to u, i.e. lam^T (A_T u) up to the
 // factor k_T.
 __global__ void __launch_bounds__(CTA) k_grad(int N, const int* __restrict__ rs, int64_t block,
-                                              const double* __restrict__ u, const double* __restrict__ lam,
+                                              const double* u, const double* lam,
                                               const double* __restrict__ W, const Tile* __restrict__ tiles,
-                                              double* __restrict__ partial) {
+                                              double* partial) {
   launch_next();
   after_previous();
   __shared__ double sh[32];
@@ -2568,7 +2595,7 @@ __global__ void __launch_bounds__(CTA) k_grad(int N, const int* __restrict__ rs,
   if (threadIdx.x == 0 && threadIdx.y == 0) partial[(size_t)macro * gridDim.x + blockIdx.x] = s;
 }
 
-__global__ void k_reduce_per_macro(const double* __restrict__ partial, int n_per, double* __restrict__ out) {
+__global__ void k_reduce_per_macro(const double* partial, int n_per, double* out) {
   launch_next();
   after_previous();
   __shared__ double sh[33];
@@ -2582,8 +2609,8 @@ __global__ void k_reduce_per_macro(const double* __restrict__ partial, int n_per
 // Sum of the partial sums into out and, where host is given, into pinned host
 // memory with the mesh's error flag beside it: the caller waits for the stream
 // and reads them, without two copies of a few bytes behind the kernel.
-__global__ void k_reduce(const double* __restrict__ partial, int n, double* __restrict__ out, double* host,
-                         const int* __restrict__ err, int* host_err) {
+__global__ void k_reduce(const double* partial, int n, double* out, double* host,
+                         const int* err, int* host_err) {
   launch_next();
   after_previous();
   __shared__ double sh[33];
@@ -2653,12 +2680,12 @@ __device__ __forceinline__ bool grid_row(const Tile& t, const MacroGeo& g, int N
 // fs), u on the closed lattice.  The first n_if_ctas CTAs take the masters.
 __global__ void __launch_bounds__(CTA) k_import(int N, const int* __restrict__ rs, int64_t block,
                                                 const MacroGeo* __restrict__ geo, int64_t nx, int64_t ny,
-                                                const double* __restrict__ gf, const double* __restrict__ gu,
-                                                double* __restrict__ f, double* __restrict__ fs,
-                                                const double* __restrict__ winv, double* __restrict__ u,
+                                                const double* gf, const double* gu,
+                                                double* f, double* fs,
+                                                const double* __restrict__ winv, double* u,
                                                 const Tile* __restrict__ tiles, int n_tiles,
-                                                const int64_t* __restrict__ if_gid, int n_if, double* __restrict__ fI,
-                                                double* __restrict__ uI, int n_if_ctas) {
+                                                const int64_t* __restrict__ if_gid, int n_if, double* fI,
+                                                double* uI, int n_if_ctas) {
   launch_next();
   after_previous();
   if ((int)blockIdx.x < n_if_ctas) {
@@ -2675,17 +2702,23 @@ __global__ void __launch_bounds__(CTA) k_import(int N, const int* __restrict__ r
   const size_t b = (size_t)macro * block + row_base(rs, N, r.j, r.k) + r.m;
   const int CS = __ldg(rs + N + 2), top = N - r.j - r.k;
   const double w = fs ? winv[macro] : 0.0;
+  const bool row_in = gf && r.j >= 1 && r.k >= 1;
+  double xu[4], xf[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {   // all loads before the stores
+    const int i = 4 * r.m + q;
+    const int64_t g = r.gid0 + i * r.step;
+    xu[q] = gu && i <= top ? gu[g] : 0.0;
+    xf[q] = row_in && i >= 1 && i < top ? gf[g] : 0.0;
+  }
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     const int i = 4 * r.m + q;
-    if (i > top) continue;
-    const int64_t g = r.gid0 + i * r.step;
     const size_t o = b + (size_t)((i + 2 * r.j + 3 * r.k) & 3) * CS;
-    if (gu) u[o] = gu[g];
-    if (gf && i >= 1 && r.j >= 1 && r.k >= 1 && i < top) {
-      const double x = gf[g];
-      f[o] = x;
-      if (fs) fs[o] = x * w;
+    if (gu && i <= top) u[o] = xu[q];
+    if (row_in && i >= 1 && i < top) {
+      f[o] = xf[q];
+      if (fs) fs[o] = xf[q] * w;
     }
   }
 }
@@ -2693,8 +2726,8 @@ __global__ void __launch_bounds__(CTA) k_import(int N, const int* __restrict__ r
 // The interior nodes of the blocks and the masters into the global vector g.
 __global__ void __launch_bounds__(CTA) k_export(int N, const int* __restrict__ rs, int64_t block,
                                                 const MacroGeo* __restrict__ geo, int64_t nx, int64_t ny,
-                                                const double* __restrict__ u, const double* __restrict__ uI,
-                                                double* __restrict__ g, const Tile* __restrict__ tiles, int n_tiles,
+                                                const double* u, const double* uI,
+                                                double* g, const Tile* __restrict__ tiles, int n_tiles,
                                                 const int64_t* __restrict__ if_gid, int n_if, int n_if_ctas) {
   launch_next();
   after_previous();
@@ -2708,16 +2741,21 @@ __global__ void __launch_bounds__(CTA) k_export(int N, const int* __restrict__ r
   if (!grid_row(tiles[v - macro * n_tiles], geo[macro], N, nx, ny, r) || r.j < 1 || r.k < 1) return;
   const size_t b = (size_t)macro * block + row_base(rs, N, r.j, r.k) + r.m;
   const int CS = __ldg(rs + N + 2), top = N - r.j - r.k;
+  double x[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {   // all loads before the stores
+    const int i = 4 * r.m + q;
+    x[q] = i >= 1 && i < top ? u[b + (size_t)((i + 2 * r.j + 3 * r.k) & 3) * CS] : 0.0;
+  }
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     const int i = 4 * r.m + q;
-    if (i < 1 || i >= top) continue;
-    g[r.gid0 + i * r.step] = u[b + (size_t)((i + 2 * r.j + 3 * r.k) & 3) * CS];
+    if (i >= 1 && i < top) g[r.gid0 + i * r.step] = x[q];
   }
 }
 
 template <class T>
-__global__ void k_import_if(const int64_t* __restrict__ gid, int n, const double* __restrict__ g, T* __restrict__ m) {
+__global__ void k_import_if(const int64_t* __restrict__ gid, int n, const double* g, T* m) {
   launch_next();
   after_previous();
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
@@ -2725,7 +2763,7 @@ __global__ void k_import_if(const int64_t* __restrict__ gid, int n, const double
 }
 
 template <class T>
-__global__ void k_export_if(const int64_t* __restrict__ gid, int n, const T* __restrict__ m, double* __restrict__ g) {
+__global__ void k_export_if(const int64_t* __restrict__ gid, int n, const T* m, double* g) {
   launch_next();
   after_previous();
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
@@ -2735,9 +2773,9 @@ __global__ void k_export_if(const int64_t* __restrict__ gid, int n, const T* __r
 // out[node] = (A u)_node over the copies listed for each node (the healthy
 // copies give A_I, the flux of the healthy side at an interface node).
 template <bool S7>
-__global__ void k_if_apply(int N, const int* __restrict__ rs, int64_t block, const double* __restrict__ u,
-                           const double* __restrict__ uI, const double* __restrict__ W, const int* __restrict__ cptr,
-                           const Copy* __restrict__ cps, const int* __restrict__ list, int n, double* __restrict__ out) {
+__global__ void k_if_apply(int N, const int* __restrict__ rs, int64_t block, const double* u,
+                           const double* uI, const double* __restrict__ W, const int* __restrict__ cptr,
+                           const Copy* __restrict__ cps, const int* __restrict__ list, int n, double* out) {
   launch_next();
   after_previous();
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
@@ -2748,7 +2786,7 @@ __global__ void k_if_apply(int N, const int* __restrict__ rs, int64_t block, con
   out[node] = diag * uI[node] + off;
 }
 
-__global__ void k_copy_listed(const double* __restrict__ src, double* __restrict__ dst, const int* __restrict__ idx,
+__global__ void k_copy_listed(const double* src, double* dst, const int* __restrict__ idx,
                               int n) {
   launch_next();
   after_previous();
@@ -2756,23 +2794,26 @@ __global__ void k_copy_listed(const double* __restrict__ src, double* __restrict
   if (q < n) dst[idx[q]] = src[idx[q]];
 }
 
-__global__ void k_scale_blocks(const double* __restrict__ f, const double* __restrict__ winv,
-                               double* __restrict__ out, int n_macro, int64_t block) {
-  launch_next();
-  after_previous();
-  const int64_t total = (int64_t)n_macro * block;
+__device__ __forceinline__ void scale_all(const double* __restrict__ f, const double* __restrict__ winv,
+                                          double* __restrict__ out, int64_t total, int64_t block) {
   for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < total; q += (int64_t)gridDim.x * blockDim.x)
     out[q] = f[q] * winv[q / block];
 }
+__global__ void k_scale_blocks(const double* f, const double* __restrict__ winv, double* out, int n_macro,
+                               int64_t block) {
+  launch_next();
+  after_previous();
+  scale_all(f, winv, out, (int64_t)n_macro * block, block);
+}
 
-__global__ void k_set_masters_zero(double* __restrict__ uI, const int* __restrict__ ids, int n) {
+__global__ void k_set_masters_zero(double* uI, const int* __restrict__ ids, int n) {
   launch_next();
   after_previous();
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q < n) uI[ids[q]] = 0.0;
 }
 
-__global__ void k_restore(double* __restrict__ u, const double* __restrict__ uI, const int64_t* __restrict__ off,
+__global__ void k_restore(double* u, const double* uI, const int64_t* __restrict__ off,
                           const int* __restrict__ master, int n) {
   launch_next();
   after_previous();
@@ -2781,7 +2822,7 @@ __global__ void k_restore(double* __restrict__ u, const double* __restrict__ uI,
 }
 
 template <class T>
-__global__ void k_zero_blocks(T* __restrict__ u, int64_t block, const int* __restrict__ act) {
+__global__ void k_zero_blocks(T* u, int64_t block, const int* __restrict__ act) {
   launch_next();
   after_previous();
   T* b = u + (size_t)act[blockIdx.y] * block;
@@ -2790,7 +2831,7 @@ __global__ void k_zero_blocks(T* __restrict__ u, int64_t block, const int* __res
 }
 
 template <class T>
-__global__ void k_zero_list(T* __restrict__ uI, const int* __restrict__ list, int n) {
+__global__ void k_zero_list(T* uI, const int* __restrict__ list, int n) {
   launch_next();
   after_previous();
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
@@ -3663,7 +3704,9 @@ cudaError_t gs_colour(const LevelArgs& L, const ProbArgs& p, T* u, T* uI, const 
   }
   const Units g = units(n, L.n_tiles_int, p.n_act);
   if (g.total == 0) return cudaSuccess;
-  auto kern = seven_point ? k_gs<T, true> : k_gs<T, false>;
+  const bool dep = dep_size(p, g.total) <= DEP_MAX_CTAS;
+  auto kern = seven_point ? (dep ? k_gs<T, true, true> : k_gs<T, true, false>)
+                          : (dep ? k_gs<T, false, true> : k_gs<T, false, false>);
   const unsigned grid = resident_grid((const void*)kern, g.total, p.grid_cap);
   if (ev_begin) cudaEventRecord(ev_begin, s);
   ++g_kernel_launches;
@@ -3756,10 +3799,14 @@ cudaError_t residual(const LevelArgs& L, const ProbArgs& p, const T* u, const T*
                double*, int*, int, int, int);
   const int skip_lo = skip >= 0 && skip < 4 ? p.col_off[skip] : 0;
   const int skip_hi = skip >= 0 && skip < 4 ? p.col_off[skip + 1] : 0;
+  const bool dep = dep_size(p, g.total) <= DEP_MAX_CTAS;
+  if (write_r && norm) return cudaErrorNotSupported;   // no caller wants both
   if (seven_point)
-    kern = write_r ? (norm ? k_res<T, true, true, true> : k_res<T, true, true, false>) : k_res<T, true, false, true>;
+    kern = write_r ? (dep ? k_res<T, true, true, false, true> : k_res<T, true, true, false, false>)
+                   : (dep ? k_res<T, true, false, true, true> : k_res<T, true, false, true, false>);
   else
-    kern = write_r ? (norm ? k_res<T, false, true, true> : k_res<T, false, true, false>) : k_res<T, false, false, true>;
+    kern = write_r ? (dep ? k_res<T, false, true, false, true> : k_res<T, false, true, false, false>)
+                   : (dep ? k_res<T, false, false, true, true> : k_res<T, false, false, true, false>);
   const unsigned grid = resident_grid((const void*)kern, g.total, p.grid_cap);
   if (n_part && norm) *n_part = (int)grid;
   ++g_kernel_launches;
@@ -3806,9 +3853,11 @@ cudaError_t restrict_to(const LevelArgs& C, const LevelArgs& F, const ProbArgs& 
         C.cptr, C.cps, C.cp_off, pc.free_if, n, pc.gather, pc.zero_off, pc.n_zero, n_if_ctas, n_vol_ctas);
     return cudaGetLastError();
   }
-  const unsigned grid = resident_grid((const void*)k_restrict<T>, g.total, pc.grid_cap);
+  const int64_t size = dep_size(pc, g.total);
+  auto kern = size <= DEP_MAX_CTAS ? k_restrict<T, true> : k_restrict<T, false>;
+  const unsigned grid = resident_grid((const void*)kern, g.total, pc.grid_cap);
   ++g_kernel_launches;
-  launch(dep_size(pc, g.total), k_restrict<T>, grid, cta_shape(), 0, s, C.N, C.rs, C.block, fc, fIc, uc, uIc, F.N, F.rs, F.block, rf, C.tiles_int,
+  launch(size, kern, grid, cta_shape(), 0, s, C.N, C.rs, C.block, fc, fIc, uc, uIc, F.N, F.rs, F.block, rf, C.tiles_int,
                                              C.n_tiles_int, pc.act, pc.n_act, C.cptr, C.cps, C.cp_off, pc.free_if, n,
                                              pc.gather, pc.zero_off, pc.n_zero, g.n_if_units, pc.sched);
   return cudaGetLastError();
@@ -3865,9 +3914,11 @@ cudaError_t prolong_add(const LevelArgs& F, const LevelArgs& C, const ProbArgs& 
         pf.n_act, F.cptr, F.cps, F.cp_off, pf.free_if, n, if_lo, if_hi, n_if_ctas, n_vol_ctas);
     return cudaGetLastError();
   }
-  const unsigned grid = resident_grid((const void*)k_prolong<T>, g.total, pf.grid_cap);
+  const int64_t size = dep_size(pf, g.total);
+  auto kern = size <= DEP_MAX_CTAS ? k_prolong<T, true> : k_prolong<T, false>;
+  const unsigned grid = resident_grid((const void*)kern, g.total, pf.grid_cap);
   ++g_kernel_launches;
-  launch(dep_size(pf, g.total), k_prolong<T>, grid, cta_shape(), 0, s, F.N, F.rs, F.block, uf, uIf, C.N, C.rs, C.block, uc, F.tiles_int,
+  launch(size, kern, grid, cta_shape(), 0, s, F.N, F.rs, F.block, uf, uIf, C.N, C.rs, C.block, uc, F.tiles_int,
                                             F.n_tiles_int, pf.act, pf.n_act, F.cptr, F.cps, F.cp_off, pf.free_if, n,
                                             g.n_if_units, pf.sched, skip, if_lo, if_hi);
   return cudaGetLastError();
