@@ -21,7 +21,7 @@ CSRC = os.path.join(HERE, "csrc")
 OUT_DIR = os.path.join(HERE, "_lib")
 LIB = os.path.join(OUT_DIR, "libhhg.so")
 SOURCES = ["mesh.cpp", "kernels.cu", "general.cu", "api.cu"]
-HEADERS = ["hhg_internal.h", "hhg_kernels.h"]
+HEADERS = ["hhg_internal.h", "hhg_kernels.h", "cg_scalar.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC,-O3,-ffp-contract=off", "--expt-relaxed-constexpr",
          "-I" + os.path.join(ROOT, "include")]

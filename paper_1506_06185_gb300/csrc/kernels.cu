@@ -44,6 +44,8 @@
 
 #include "hhg_kernels.h"
 
+#include "cg_scalar.cuh"
+
 namespace hhg {
 
 std::atomic<long long> g_kernel_launches{0};
@@ -2112,56 +2114,13 @@ __device__ __forceinline__ double cg_rows_sum(int n, double* buf, F&& body) {
   return warp_sum_xor(buf[lane]);
 }
 
-// 1 / b, about one unit in the last place: the hardware's reciprocal
-// approximation y and one third-order step y (1 + e + e^2), e = 1 - b y
-// (Halley's iteration for 1 / b).  Three dependent FP64 operations of 68
-// clocks each where the IEEE division takes 590 clocks of latency; x and r
-// move by the same step, so its rounding only turns the search direction.
-// Operands near the ends of the exponent range take the IEEE division.
-__device__ __noinline__ double cg_recip_ieee(double b) { return 1.0 / b; }
-__device__ __forceinline__ double cg_recip(double b) {
-  const uint32_t e = ((uint32_t)__double2hiint(b) >> 20) & 0x7ffu;
-  if (e - 64u > 0x7ffu - 128u) return cg_recip_ieee(b);
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(b));
-  double d = fma(-b, y, 1.0);
-  d = fma(d, d, d);
-  return fma(y, d, y);
-}
-
-// The test sqrt(rr) > thr, set up once for a thr: rr (>= 0, or not a number) is
-// compared as an integer with thr^2 (1 +- 1e-14), and only between the two, or
-// where thr^2 is near the ends of the exponent range, the square root (650
-// clocks) is taken.
-struct CgTest {
-  double thr;
-  long long lo, hi;
-};
-__device__ __forceinline__ CgTest cg_test(double thr) {
-  CgTest t{thr, 0, 0x7ff0000000000000ll};
-  const double t2 = thr * thr;
-  if (t2 > 1e-280 && t2 < 1e280) {
-    t.lo = __double_as_longlong(t2 * (1.0 - 1e-14));
-    t.hi = __double_as_longlong(t2 * (1.0 + 1e-14));
-  }
-  return t;
-}
-__device__ __noinline__ bool cg_above_sqrt(double rr, double thr) { return sqrt(rr) > thr; }
-__device__ __forceinline__ bool cg_above(double rr, const CgTest& t) {
-  const long long b = __double_as_longlong(rr);
-  if (b > t.hi && b < 0x7ff0000000000000ll) return true;
-  if (b < t.lo) return false;
-  return cg_above_sqrt(rr, t.thr);
-}
-
 // CG on the compact free nodes of the coarsest level from x = 0 until
 // ||r|| <= rtol ||b|| or maxit iterations, with z = r, or, given the
 // reciprocal diagonal, z = r / diag (Jacobi preconditioning; below r.r stands
 // for r.z, the stopping test keeps r.r).  The direction's image s = A p is
 // carried along, s <- A r + beta s, so that the product A r does not wait for
 // beta.  One iteration: p.s, alpha = r.r / p.s, x += alpha p, r -= alpha s,
-// r.r, beta = r.r / old r.r (times the reciprocal, formed beside the critical
-// path), p <- r + beta p, s <- A r + beta s.  A row's product is summed in two
+// r.r, beta = r.r / old r.r (the reciprocal formed beside the critical path), p <- r + beta p, s <- A r + beta s.  A row's product is summed in two
 // chains, even and odd entries.
 //
 // One CTA of CG_THREADS threads; x, r, p and s live in shared or in global
@@ -2202,6 +2161,22 @@ __device__ __forceinline__ void cg_one_cta(int n, const int* rowptr, const int* 
     return b * z(q);
   });
   double rr = dinv ? squares() : rz;
+  double back = 1.0;
+  if (!cg_in_range(rr)) {   // cg_shift
+    uint32_t m = 0;
+    for (int q = t; q < n; q += CG_THREADS) m = max(m, cg_exponent(r[q]));
+    m = __reduce_max_sync(0xffffffffu, m);
+    __syncthreads();   // the totals have been read
+    if ((t & 31) == 0) red[t >> 5] = (double)m;
+    __syncthreads();
+    for (int w = 0; w < CG_WARPS; ++w) m = max(m, (uint32_t)red[w]);
+    const double up = cg_shift(m);
+    back = 1.0 / up;
+    for (int q = t; q < n; q += CG_THREADS) r[q] *= up;
+    __syncthreads();
+    rz = cg_rows_sum(n, red, [&](int q) { return r[q] * z(q); });
+    rr = dinv ? squares() : rz;
+  }
   const double bnorm = sqrt(rr);
   const CgTest test = cg_test(rtol * bnorm);
   int it = 0;
@@ -2234,7 +2209,7 @@ __device__ __forceinline__ void cg_one_cta(int n, const int* rowptr, const int* 
     ++it;
   }
   for (int q = t; q < n; q += CG_THREADS) {
-    const T v = (T)x[q];
+    const T v = (T)(x[q] * back);
     for (int e = uptr[q]; e < uptr[q + 1]; ++e) u[udst[e]] = v;
     if (umaster[q] >= 0) uI[umaster[q]] = v;
   }
@@ -2464,20 +2439,38 @@ __global__ void __launch_bounds__(NB > 0 ? CG_THREADS + 32 : 1024) k_cg_cluster(
   double* gw = gs + (NB > 0 ? 0 : (size_t)A.n);
   after_previous();
   barrier();   // every CTA of the cluster runs before its memory is written
-  each_sum(peer0, [&](int i, int g, int q) {
-    double v = 0.0;
-    if (q >= 0) {
-      const int64_t src = A.fsrc[q];
-      v = src >= 0 ? (double)f[src] : (double)fI[-1 - src];
-      if (NB == 0) gx[q] = 0.0;
+  double up = 1.0;   // cg_shift; all CTAs decide alike
+  for (bool first = true;; first = false) {
+    each_sum(peer0, [&](int i, int g, int q) {
+      double v = 0.0;
+      if (q >= 0) {
+        const int64_t src = A.fsrc[q];
+        v = up * (src >= 0 ? (double)f[src] : (double)fI[-1 - src]);
+        if (NB == 0) gx[q] = 0.0;
+      }
+      if (NB > 0) rr_[i] = v;
+      const double zv = z(i, v);
+      sr[slot(i, g)] = zv;
+      return v * zv;
+    });
+    squares();
+    barrier();   // b.b summed; every r entry written
+    if (!first || cg_in_range(cg_total(jac ? sum2 : sum0, nb))) break;
+#pragma unroll
+    for (int i = 0; i < ni; ++i) {
+      if (!mine(i)) continue;
+      uint32_t m = NB > 0 ? cg_exponent(rr_[NB > 0 ? i : 0]) : 0;
+      if constexpr (NB == 0)
+        for (int g = 0; g < 1 << sh; ++g) m = max(m, cg_exponent(sr[slot(i, g)]));
+      m = __reduce_max_sync(0xffffffffu, m);
+      const int b = (warp + i * W) * (int)C + (int)rank;
+      if (b < nb && lane < (int)C) cluster_store(peer1 + (uint32_t)b * 8, (double)m);
     }
-    if (NB > 0) rr_[i] = v;
-    const double zv = z(i, v);
-    sr[slot(i, g)] = zv;
-    return v * zv;
-  });
-  squares();
-  barrier();   // b.b summed; every r entry written
+    barrier();   // the blocks' exponents are written, the sums have been read
+    uint32_t m = 0;
+    for (int b = lane; b < nb; b += 32) m = max(m, (uint32_t)sum1[b]);
+    up = cg_shift(__reduce_max_sync(0xffffffffu, m));
+  }
   double rz = 0.0, rr = 0.0, inv = 0.0;   // scalar warp
   CgTest test{0.0, 0, 0};
   bool any = false;
@@ -2544,9 +2537,10 @@ __global__ void __launch_bounds__(NB > 0 ? CG_THREADS + 32 : 1024) k_cg_cluster(
     ++it;
     barrier();   // r.r summed; every r entry written
   }
+  const double back = 1.0 / up;
   each([&](int i, int, int q) {
     if (q < 0) return;
-    const T v = (T)(NB > 0 ? xr[i] : gx[q]);
+    const T v = (T)((NB > 0 ? xr[i] : gx[q]) * back);
     for (int e = A.uptr[q]; e < A.uptr[q + 1]; ++e) u[A.udst[e]] = v;
     if (A.umaster[q] >= 0) uI[A.umaster[q]] = v;
   });
@@ -4020,6 +4014,7 @@ const double* cg_precond(const DevProblem& p, double rtol, int maxit) {
 template <class T>
 cudaError_t coarse_cg(const DevProblem& p, const T* f, const T* fI, T* u, T* uI, double rtol, int maxit,
                       cudaStream_t s, double* work) {
+  rtol = std::max(rtol, CG_RTOL_MIN);
   if (g_rec) {
     if (p.n_cg == 0) return cudaSuccess;
     BOp op = new_op<T>(BOP_CG);
