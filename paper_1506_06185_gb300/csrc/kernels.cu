@@ -2068,8 +2068,9 @@ __device__ __forceinline__ double warp_sum_xor(double v) {
 // at a time.  Their four trees run as one: after the step over 16 lanes each
 // half of the warp holds two of them, after the step over 8 each quarter one,
 // so four blocks cost six additions instead of twenty (one CTA is bound by the
-// FP64 pipe: with a tree per block the persistent batch with a 3375-row coarse
-// problem took 248 ms instead of 210).  Quarter e of the warp ends with block
+// FP64 pipe, 2 lanes a clock and about 17 operations a row and iteration: a
+// cycle of 4x4x4 sub-cubes refined 3 times, 3375 coarse rows, takes 3.45 ms in
+// the executor, 4.45 with a tree per block).  Quarter e of the warp ends with block
 // e's sum, the same bits as warp_sum_xor, and holds bucket w + 8 e.
 __device__ __forceinline__ double warp_sum4(const double (&v)[4]) {
   const bool h16 = (threadIdx.x & 16) != 0, h8 = (threadIdx.x & 8) != 0;
@@ -3164,8 +3165,12 @@ __device__ void unit_prolong(const BOp& op, int unit, int (*s_pre2)[33], int* s_
 }
 
 // Unit of the FP64 residual handed to the FP32 cycle (k_res_f32, no norm).
+// This unit and the coarse CG are called, not inlined: the executor has 48
+// registers, and what these two hold was spilled in the Gauss-Seidel loops (a
+// mixed 4x4x4 global task of refinement 7 with 64 recovery tasks 235.4 -> 211.8
+// ms, the global task alone first 212.2 -> 188.7; small batches as before).
 template <bool S7>
-__device__ void unit_res_f32(const BOp& op, int unit, int (*s_pre2)[33], int* s_pre_tot) {
+__device__ __noinline__ void unit_res_f32(const BOp& op, int unit, int (*s_pre2)[33], int* s_pre_tot) {
   const LevelArgs& L = op.L;
   const ProbArgs& p = op.P;
   const int N = L.N;
