@@ -1475,14 +1475,15 @@ __global__ void __launch_bounds__(CTA) k_res_flat(int N, const int* __restrict__
     const int j = (int)(d >> 20), k = (int)((d >> 10) & 1023u), g = (int)(d & 1023u);
     const T* w = W + (size_t)macro * 16 * NDIR;
     const size_t mb = (size_t)macro * block;
-    const Slice sc = slice_consts(rs, N, k);
+    // slice_consts inside each branch: before it the constants stay live through
+    // both, 48 registers instead of 40 and five CTAs per SM instead of six
     if constexpr (S7) {
       const T wr[11] = {w[0], w[1], w[2], w[3], T(0), T(0), T(0), T(0), w[8], w[9], w[10]};
-      if (c == skip) res_group7<T, WRITE, NORM, true>(sc, N, j, g, c, u + mb, f + mb, r + mb, wr, ss);
-      else res_group7<T, WRITE, NORM, false, !DEP>(sc, N, j, g, c, u + mb, f + mb, r + mb, wr, ss);
+      if (c == skip) res_group7<T, WRITE, NORM, true>(slice_consts(rs, N, k), N, j, g, c, u + mb, f + mb, r + mb, wr, ss);
+      else res_group7<T, WRITE, NORM, false, !DEP>(slice_consts(rs, N, k), N, j, g, c, u + mb, f + mb, r + mb, wr, ss);
     } else {
-      if (c == skip) res_group15<T, WRITE, NORM, true>(sc, N, j, g, c, u + mb, f + mb, r + mb, w, ss);
-      else res_group15<T, WRITE, NORM, false, !DEP>(sc, N, j, g, c, u + mb, f + mb, r + mb, w, ss);
+      if (c == skip) res_group15<T, WRITE, NORM, true>(slice_consts(rs, N, k), N, j, g, c, u + mb, f + mb, r + mb, w, ss);
+      else res_group15<T, WRITE, NORM, false, !DEP>(slice_consts(rs, N, k), N, j, g, c, u + mb, f + mb, r + mb, w, ss);
     }
   }
   if (NORM) {
