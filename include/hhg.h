@@ -419,6 +419,11 @@ int hhg_set_launch_limit(hhg_mesh* mesh, int max_ctas);
  * Allocates and frees a small device buffer; synchronises. */
 int hhg_measure_fp64_peak(double* tflops);
 int hhg_walk_counts(hhg_mesh* mesh, int64_t* counts);
+/* hhg_flat_levels: flat[l] = 1 where the cycles' launches on level l (coarsest
+ * first; on the coarsest only the restriction onto it) take the flat kernels as
+ * the mesh is set now, 0 where they take the tile kernels (the streaming
+ * kernel, where switched on, replaces either in the 7-point sweeps). */
+int hhg_flat_levels(const hhg_mesh* mesh, int* flat);
 
 /* Kernel options (implementation knobs, not part of the method).
  * hhg_set_streaming: enable or disable (default) the streaming Gauss-Seidel

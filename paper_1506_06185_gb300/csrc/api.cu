@@ -2159,6 +2159,12 @@ int hhg_walk_counts(hhg_mesh* m, int64_t* counts) {
   return HHG_OK;
 }
 
+int hhg_flat_levels(const hhg_mesh* m, int* flat) {
+  if (!m || !flat) return fail(HHG_ERR_ARG, "null argument");
+  for (int l = 0; l < (int)m->host.lv.size(); ++l) flat[l] = flat_on(largs(m, l), pargs(m->global, l)) ? 1 : 0;
+  return HHG_OK;
+}
+
 int hhg_measure_fp64_peak(double* tflops) {
   if (!tflops) return fail(HHG_ERR_ARG, "null argument");
   int dev = 0, sms = 0;

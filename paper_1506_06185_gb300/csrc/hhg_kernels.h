@@ -117,6 +117,10 @@ cudaError_t coarse_cg(const DevProblem& p, const T* f, const T* fI, T* u, T* uI,
 cudaError_t reduce_partials(const double* partial, int n, double* out, cudaStream_t s, double* host = nullptr,
                             const int* err = nullptr, int* host_err = nullptr);
 
+// Whether a level's launches take the flat kernels: switched on, or left to the
+// default, which a launch limit turns into the tile kernels it limits.
+bool flat_on(const LevelArgs& L, const ProbArgs& p);
+
 // FP64 FMA throughput probe: `blocks` CTAs of 256 threads, 8 x iters FMAs per
 // thread; out holds blocks * 256 doubles.
 cudaError_t fma_probe(double* out, int blocks, int iters, cudaStream_t s);

@@ -3639,9 +3639,9 @@ cudaError_t launch_gs_stream(const LevelArgs& L, const ProbArgs& p, T* u, T* uI,
   return cudaGetLastError();
 }
 
-// Whether a level's launches take the flat kernels: switched on (1), or left to
-// the default (2), which a launch limit turns into the tile kernels it limits.
-bool flat_on(const LevelArgs& L, const ProbArgs& p) { return L.gs_flat == 1 || (L.gs_flat == 2 && p.grid_cap == 0); }
+bool flat_on(const LevelArgs& L, const ProbArgs& p) {
+  return L.gs_flat == FLAT_ON || (L.gs_flat == FLAT_AUTO && p.grid_cap == 0);
+}
 
 template <class T>
 cudaError_t gs_colour(const LevelArgs& L, const ProbArgs& p, T* u, T* uI, const T* f, const T* fI, const T* W,

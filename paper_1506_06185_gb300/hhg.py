@@ -30,7 +30,8 @@ EXPORTS = ["hhg_mesh_create", "hhg_mesh_destroy", "hhg_mesh_info", "hhg_mesh_byt
            "hhg_autotune", "hhg_batch_create", "hhg_batch_launch", "hhg_batch_destroy",
            "hhg_batch_launch_persistent", "hhg_batch_info", "hhg_batch_set_priority", "hhg_recover_dn",
            "hhg_mesh_create_general", "hhg_set_launch_limit", "hhg_walk_counts", "hhg_set_streaming",
-           "hhg_set_wait_limit", "hhg_measure_fp64_peak", "hhg_profile_breakdown", "hhg_set_flat_gs"]
+           "hhg_set_wait_limit", "hhg_measure_fp64_peak", "hhg_profile_breakdown", "hhg_set_flat_gs",
+           "hhg_flat_levels"]
 
 
 class hhg_mesh_desc(C.Structure):
@@ -96,6 +97,7 @@ def load_library(path: str = LIB_PATH) -> C.CDLL:
         "hhg_set_streaming": ([P, C.c_int], C.c_int),
         "hhg_set_wait_limit": ([P, C.c_int], C.c_int),
         "hhg_set_flat_gs": ([P, C.c_int], C.c_int),
+        "hhg_flat_levels": ([P, C.POINTER(C.c_int)], C.c_int),
         "hhg_measure_fp64_peak": ([C.POINTER(C.c_double)], C.c_int),
         "hhg_profile_breakdown": ([P, C.POINTER(C.c_double), C.c_int], C.c_int),
         "hhg_vcycle_noalloc": ([P, C.c_int, C.c_int, P], C.c_int),
@@ -432,6 +434,13 @@ def hhg_set_wait_limit(h, tries):
     """tries >= 0: at most that many tries per bounded device wait (0: every
     wait runs out at once); tries < 0: the default."""
     return _check(lib().hhg_set_wait_limit(h, int(tries)))
+
+
+def hhg_flat_levels(h, n_levels):
+    """Whether the launches of each level (coarsest first) take the flat kernels."""
+    c = (C.c_int * int(n_levels))()
+    _check(lib().hhg_flat_levels(h, c))
+    return [bool(v) for v in c]
 
 
 def hhg_walk_counts(h):
