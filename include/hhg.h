@@ -278,8 +278,9 @@ int hhg_grad_coeff(hhg_mesh* mesh, const double* u, const double* lam, double* g
  * the sweeps smooth) and, on precision-32 meshes, also on the FP32 arrays,
  * and keeps for that level the shape with the least total time; it then
  * times the flat Gauss-Seidel kernel
- * (hhg_set_flat_gs) and keeps it for the level's sweeps if it is faster
- * still (the residual and transfer kernels keep the chosen tiles).
+ * (hhg_set_flat_gs) and, if it is faster still, leaves the level to the flat
+ * kernels (sweeps, residual and transfers), except while a launch limit is
+ * set (hhg_set_launch_limit), which selects the tile kernels.
  * chosen (may be NULL, one int per level, coarsest first) receives the index
  * c of the chosen tile shape, or c + 4 when the level's Gauss-Seidel sweeps
  * use the flat kernel (-1 for the coarsest level, which is not smoothed).
@@ -390,9 +391,10 @@ int hhg_vcycle_noalloc(hhg_mesh* mesh, int pre, int post, void* stream);
  * each kernel of a CUDA graph the library replays (batched recovery, the
  * later cycles of a local recovery) counts as one launch per replay, kernels
  * recorded while capturing such a graph do not count.
- * hhg_set_launch_limit: at most max_ctas CTAs per level-wide launch of the
- * tile kernels (0, the default: as many as the GPU holds at once; the flat
- * kernels launch one CTA per 256 items and are not limited).  A level-wide launch walks its
+ * hhg_set_launch_limit: at most max_ctas CTAs per level-wide launch (0, the
+ * default: as many as the GPU holds at once).  A limit selects the tile kernels
+ * on every level but those that hhg_set_flat_gs switched on, whose flat kernels
+ * launch one CTA per 256 items and are not limited.  A level-wide launch walks its
  * work units (interface chunks, then volume tiles) with a grid stride when
  * it has fewer than 4 units per CTA, and otherwise hands the units out
  * through a per-problem counter (the dynamic walk of large launches, where
@@ -432,7 +434,7 @@ int hhg_flat_levels(const hhg_mesh* mesh, int* flat);
  * producer warp staging the two neighbour colours and the right-hand side of
  * each slice in shared memory with bulk asynchronous copies on mbarriers for
  * eight consumer warps; disabled, each level uses the row-pair tile kernel or,
- * where switched on (hhg_set_flat_gs, hhg_autotune), the flat kernel.  All
+ * by default or where switched on (hhg_set_flat_gs), the flat kernel.  All
  * give the same iterate bit for bit (the streaming kernel is the slowest of
  * the three on GB300).  Drops the captured recovery-cycle graph.
  * hhg_set_wait_limit: the streaming kernel's waits on its mbarriers are bounded

@@ -1313,15 +1313,16 @@ int tune_level(hhg_mesh* m, int l, int reps, cudaStream_t s, int* best_out) {
   tb.tiles_int = dev[best];
   tb.n_tiles_int = ndev[best];
   *best_out = best;
-  // the flat Gauss-Seidel kernel against the best tile shape; the level's
-  // other kernels keep the tiles either way
+  // the flat Gauss-Seidel kernel against the best tile shape; the winner also
+  // gives the level's residual and transfers their form.  A flat level is left
+  // in the default mode, in which a launch limit selects the tile kernels.
   if (flat_fits(m, l)) {
     HHG_TRY(set_flat(m, l, FLAT_ON));
     float ms = 0.f, ms32 = 0.f;
     HHG_TRY(time_smooth<double>(m, m->d64, l, reps, s, a, b, &ms));
     if (m->precision == 32) HHG_TRY(time_smooth<float>(m, m->d32, l, reps, s, a, b, &ms32));
     if (ms + ms32 < best_ms) *best_out = best + N_TUNE_CAND;
-    else HHG_TRY(set_flat(m, l, FLAT_OFF));
+    HHG_TRY(set_flat(m, l, ms + ms32 < best_ms ? FLAT_AUTO : FLAT_OFF));
   }
   // the other candidates' tiles and the level's previous tiles are unused now
   std::vector<void*> unused;

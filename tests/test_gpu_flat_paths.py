@@ -61,6 +61,26 @@ def test_flat_and_tile_kernels_alike(hhg, sub, R, mesh_kw, call):
         assert len(hf) == len(ht) and np.abs(np.array(hf) - ht).max() <= 1e-12 * hf[0], limit
 
 
+@pytest.mark.parametrize("sub,R,mesh_kw", [((2, 2, 1), 5, {}), ((2, 1, 2), 5, dict(affine=SHEAR))])
+def test_launch_limit_on_a_tuned_mesh(hhg, sub, R, mesh_kw):
+    M = hhg.Mesh(sub, R, **mesh_kw)
+    f, u0 = I.random_load(sub, R, seed=22), I.initial_guess(sub, R)
+    M.set_problem(f, u0)
+    M.vcycle()
+    u = M.get_solution()
+    hhg.hhg_autotune(M.h, R - 1)
+    tuned = hhg.hhg_flat_levels(M.h, R - 1)
+    hhg.hhg_set_launch_limit(M.h, 2)
+    assert not any(hhg.hhg_flat_levels(M.h, R - 1))
+    before = hhg.hhg_walk_counts(M.h)[0]
+    M.set_problem(f, u0)
+    M.vcycle()
+    assert np.array_equal(M.get_solution(), u) and hhg.hhg_walk_counts(M.h)[0] >= before + 24
+    hhg.hhg_set_launch_limit(M.h, 0)
+    assert hhg.hhg_flat_levels(M.h, R - 1) == tuned
+    M.close()
+
+
 def test_switch_off_and_on(hhg):
     M = hhg.Mesh((2, 1, 1), 4)
     hhg.hhg_set_flat_gs(M.h, False)
