@@ -789,10 +789,13 @@ bool build_general_if_tables(const HostMesh& m, int l, const std::vector<int>& f
       for (int q = q0; q < q1; ++q) {
         const std::vector<Ent>& E = ent[q - q0];
         const Copy& own = copies[cptr[free_if[q]]];
+        // padding reads a neighbour, not the node itself, whose old value the
+        // update does not use (times 0 it would keep infinities and NaN alive)
+        const uint32_t pad = E.empty() ? offset(own.macro, own.i, own.j, own.k) : E[0].off;
         ptr[q] = (uint32_t)(base + (q - q0));
         len[q] = (int)longest;
         for (size_t e = 0; e < longest; ++e) {
-          nb[ptr[q] + 32 * e] = e < E.size() ? E[e].off : offset(own.macro, own.i, own.j, own.k);
+          nb[ptr[q] + 32 * e] = e < E.size() ? E[e].off : pad;
           w[ptr[q] + 32 * e] = e < E.size() ? E[e].w : 0.0;
         }
       }
