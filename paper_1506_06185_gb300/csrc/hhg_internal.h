@@ -177,6 +177,8 @@ struct HostLevel {
   std::vector<unsigned char> if_colour, if_dirichlet;   // general meshes: if_colour
                                       // holds the interface smoother class
   int n_if_classes = 0;               // general meshes: number of interface classes
+  std::vector<int> surf;              // general meshes: interface node at every surface node
+                                      // of every macro (surf_index)
   std::vector<double> W;              // [n_macro][16][15] stencil weights
   std::vector<Tile> tiles_int;        // row-pair tiles of the volume interior
   std::vector<Tile> tiles_all;        // tiles covering the closed lattice
@@ -185,6 +187,17 @@ struct HostLevel {
   std::vector<StreamTile> tiles_stream32;  // the same for the FP32 cycles (wider bands)
   int stream_band32 = 0;
 };
+
+// Position in HostLevel::surf of surface node (i, j, k) of a macro: four faces
+// of (N + 1)(N + 2) / 2 entries each, a node of several faces in the first of
+// them; -1 for a volume node.
+inline int64_t surf_index(int N, int macro, int i, int j, int k) {
+  const int mask = node_class(i, j, k, N);
+  if (mask == 0) return -1;
+  const int face = mask & 1 ? 0 : mask & 2 ? 1 : mask & 4 ? 2 : 3;
+  const int a = face == 2 ? j : i, b = face == 0 || face == 3 ? j : k;
+  return ((int64_t)macro * 4 + face) * ((int64_t)(N + 1) * (N + 2) / 2) + ((int64_t)a * (2 * N + 3 - a)) / 2 + b;
+}
 
 struct HostMesh {
   int sub[3] = {0, 0, 0};

@@ -741,15 +741,8 @@ bool build_general_if_tables(const HostMesh& m, int l, const std::vector<int>& f
   auto offset = [&](int t, int i, int j, int k) {
     return (uint32_t)((int64_t)t * L.block + lidx(L.SL.data(), N, i, j, k));
   };
-  // interface node at every block offset (-1: a volume node)
-  std::vector<int> node_at((size_t)m.n_macro * L.block, -1);
-  for (int q = 0; q < L.n_if; ++q)
-    for (int c = L.if_cptr[q]; c < L.if_cptr[q + 1]; ++c) {
-      const Copy& cp = L.if_copy[c];
-      node_at[offset(cp.macro, cp.i, cp.j, cp.k)] = q;
-    }
   struct Ent {
-    int64_t id;   // node, or n_if + offset of a volume node
+    int node;   // interface node, -1: a volume node
     double w;
     uint32_t off;
   };
@@ -766,17 +759,20 @@ bool build_general_if_tables(const HostMesh& m, int l, const std::vector<int>& f
         E.clear();
         for (int x = cptr[free_if[q]]; x < cptr[free_if[q] + 1]; ++x) {
           const Copy& cp = copies[x];
+          const size_t n_other = E.size();   // a node met again is one of an earlier copy's
           const double* wm = &L.W[((size_t)cp.macro * 16 + node_class(cp.i, cp.j, cp.k, N)) * NDIR];
           diag[q] += wm[0];
           for (int d = 1; d < NDIR; ++d) {
             int di, dj, dk;
             dir_ijk(d, di, dj, dk);
             if (wm[d] == 0.0 || !in_lattice(cp.i + di, cp.j + dj, cp.k + dk, N)) continue;
-            const uint32_t off = offset(cp.macro, cp.i + di, cp.j + dj, cp.k + dk);
-            const int64_t id = node_at[off] >= 0 ? node_at[off] : (int64_t)L.n_if + off;
-            auto it = std::find_if(E.begin(), E.end(), [&](const Ent& e) { return e.id == id; });
-            if (it != E.end()) it->w += wm[d];
-            else E.push_back(Ent{id, wm[d], off});
+            const int ni = cp.i + di, nj = cp.j + dj, nk = cp.k + dk;
+            const int64_t at = surf_index(N, cp.macro, ni, nj, nk);
+            const int node = at < 0 ? -1 : L.surf[at];
+            size_t e = node < 0 ? n_other : 0;
+            while (e < n_other && E[e].node != node) ++e;
+            if (e < n_other) E[e].w += wm[d];
+            else E.push_back(Ent{node, wm[d], offset(cp.macro, ni, nj, nk)});
           }
         }
         longest = std::max(longest, E.size());
@@ -1036,11 +1032,11 @@ void build_general_mesh(HostMesh& m, const double* verts, int nv, const int* tet
     L.n_if = (int)nodes.size();
     // interface classes: greedy colouring of the coupling graph of the free
     // interface nodes (lattice neighbours inside some macro), in key order
-    std::unordered_map<int64_t, int> at;               // macro * block + slot -> interface node
+    L.surf.assign((size_t)m.n_macro * 4 * ((size_t)(N + 1) * (N + 2) / 2), -1);
     for (int n = 0; n < L.n_if; ++n)
       for (int c = L.if_cptr[n]; c < L.if_cptr[n + 1]; ++c) {
         const Copy& cp = L.if_copy[c];
-        at[(int64_t)cp.macro * L.block + lidx(L.SL.data(), N, cp.i, cp.j, cp.k)] = n;
+        L.surf[surf_index(N, cp.macro, cp.i, cp.j, cp.k)] = n;
       }
     std::vector<int> cls(L.n_if, -1);
     int n_cls = 0;
@@ -1054,10 +1050,10 @@ void build_general_mesh(HostMesh& m, const double* verts, int nv, const int* tet
           dir_ijk(d, di, dj, dk);
           const int ni = cp.i + di, nj = cp.j + dj, nk = cp.k + dk;
           if (!in_lattice(ni, nj, nk, N) || node_class(ni, nj, nk, N) == 0) continue;
-          auto it = at.find((int64_t)cp.macro * L.block + lidx(L.SL.data(), N, ni, nj, nk));
-          if (it != at.end() && cls[it->second] >= 0) {
-            if (cls[it->second] >= (int)used.size()) used.resize(cls[it->second] + 1, 0);
-            used[cls[it->second]] = 1;
+          const int at = L.surf[surf_index(N, cp.macro, ni, nj, nk)];
+          if (at >= 0 && cls[at] >= 0) {
+            if (cls[at] >= (int)used.size()) used.resize(cls[at] + 1, 0);
+            used[cls[at]] = 1;
           }
         }
       }
