@@ -788,7 +788,7 @@ def extra_fifteen_point(torch, hhg, I):
     res = {"workload": "cube 2x2x2x6 macro-tets refined 8 levels under a shear (15-point stencils), random load "
                        "seed 0, fault-free FP64 solve to 1e-8",
            "seven_point": bool(seven), "ms": ms, "cycles": cyc, "final_rel_res": float(hist[-1]),
-           "gs_roofline": {"kernel": "k_gs<double, 15-point> finest level, one colour", "launches": n,
+           "gs_roofline": {"kernel": "k_gs_flat<double, 15-point> finest level, one colour", "launches": n,
                            "avg_launch_ms": avg * 1e3, "bound": "alu", "achieved_tflops": tflops,
                            "peak_tflops": peak, "frac": tflops / peak,
                            "hbm_gbs": 24.0 * n_vol / 4.0 / avg / 1e9}}

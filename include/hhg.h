@@ -237,7 +237,12 @@ typedef struct {
                              n_local = 0; DN always) */
   int mixed_precision;    /* 1: FP32 cycles inside FP64 iterative refinement
                              (needs a precision-32 mesh) */
-  double coarse_rtol;     /* coarse CG relative tolerance (0 = 1e-12) */
+  double coarse_rtol;     /* coarse CG relative tolerance (0 = 1e-12; below 1e-60 counts as 1e-60).
+                           * With the default tolerance (or a tighter one) and the default cap (or
+                           * a larger one) the CG is preconditioned with the diagonal where that
+                           * varies by more than half; a looser tolerance or a smaller cap runs
+                           * plain CG, whose iterations the caller then counts (to the same
+                           * residual it may need more of them) */
   int coarse_maxit;       /* coarse CG iteration cap (0 = 1000) */
   const hhg_fault* faults;  /* further faults (host, may be NULL), each handled
                                like the first with the same recovery */

@@ -895,9 +895,9 @@ void drop_local_graph(hhg_mesh* m) {
 // latency of Omega_F's launches counts (refined 6 times: 5.6 / 5.6 against 6.3 /
 // 2.2 ms; one macro of 3x3x3 sub-cubes in a DN solve: 16.2 against 18.2 ms).
 int overlap_beside(const hhg_mesh* m, const DevProblem& other) {
-  // CTAs of 256 vectors in one colour of one macro: about N^3 / 48 vectors
+  // CTAs of 256 vectors in one colour of one macro: about N^3 / 48 vectors (FP64)
   const int64_t N = m->host.lv.back().N, per_macro = N * N * N / (48 * 256);
-  return std::min(m->faulty.n_act, other.n_act) * per_macro <= 2432 ? 1 : 0;
+  return std::min(m->faulty.n_act, other.n_act) * per_macro <= DEP_MAX_CTAS ? 1 : 0;
 }
 
 // n cycles of the faulty problem on stream ls: the first one directly (it
@@ -1486,7 +1486,6 @@ int upload_priorities(hhg_batch* b, const std::vector<int>& prio) {
   return HHG_OK;
 }
 
-// Records every task's program and uploads it with the scheduler's counters.
 // The batch's device is current and its meshes are still there.
 int check_batch(const hhg_batch* b) {
   for (const auto& t : b->tasks)
@@ -1494,6 +1493,7 @@ int check_batch(const hhg_batch* b) {
   return b->tasks.empty() ? HHG_OK : check_device(b->tasks[0].mesh);
 }
 
+// Records every task's program and uploads it with the scheduler's counters.
 int setup_persistent(hhg_batch* b, size_t n_rec) {
   b->op_off.assign(1, 0);
   for (size_t t = 0; t < b->tasks.size(); ++t) {

@@ -358,6 +358,9 @@ struct DevLevel {
 // 231 -> 181 us, 15-point 397 -> 283 us; at 1.3e8 nodes the tile form is 12%
 // faster, its CTAs adding up many tiles each).
 constexpr int FLAT_NORM_MAX = 16384;
+// CTAs of a launch at most that may overlap its predecessor's end: two waves of
+// 8 CTAs on each of the 152 SMs.
+constexpr int64_t DEP_MAX_CTAS = 2 * 8 * 152;
 // Whether a level runs the flat kernels: off, switched on, or by default (new
 // meshes, every level the kernels can run; a launch limit selects the tile
 // kernels there).

@@ -26,8 +26,9 @@
 // One V(3,3) cycle, tile -> flat kernels: 7-point box of 3x2x1 sub-cubes
 // refined 6 times 1.41 -> 1.06 ms, 2x2x2 refined 7 times 3.96 -> 3.00 ms;
 // 15-point (sheared) refined 7 and 8 times 6.85 -> 5.35 and 35.7 -> 32.9 ms.
-// The tile kernels stay for the norms (faster there), for a launch limit, for
-// the streaming and batch forms, and for levels beyond the tables' range.
+// The tile kernels stay for norms of more than FLAT_NORM_MAX CTAs (faster
+// there), for a launch limit, for the streaming and batch forms, and for levels
+// beyond the tables' range.
 //
 // Interface work: a node's stencil is the sum of the sub-stencils of the
 // macros around it (§3.2, Fig. 4); the kernel updates the master in the
@@ -1421,7 +1422,7 @@ __global__ void __launch_bounds__(CTA, 4) k_res(int N, const int* __restrict__ r
 // stride (launched with one chunk per CTA), interface chunks spread among the
 // volume chunks; no tiles and no CTA barrier before the final norm
 // reduction.  Same arithmetic per item as k_res (res_group7), so r is the
-// same bit for bit; the norm's partial sums would follow the grid.  n_items:
+// same bit for bit; the norm's partial sums follow the grid.  n_items:
 // items per macro taken (off[4], or off[3] for a norm-only launch that skips
 // colour 3).
 template <class T, bool S7, bool WRITE, bool NORM, bool DEP>
@@ -2125,8 +2126,8 @@ __device__ __forceinline__ double cg_rows_sum(int n, double* buf, F&& body) {
 // r.r, beta = r.r / old r.r (the reciprocal formed beside the critical path), p <- r + beta p, s <- A r + beta s.  A row's product is summed in two
 // chains, even and odd entries.
 //
-// One CTA of CG_THREADS threads; x, r, p and s live in shared or in global
-// memory (4 n doubles); a row belongs to one thread throughout.  dinv: the
+// One CTA of CG_THREADS threads; x, r, p and s live in global memory (4 n
+// doubles); a row belongs to one thread throughout.  dinv: the
 // reciprocal diagonal, or null.  red: 64 doubles of shared memory.
 template <class T>
 __device__ __forceinline__ void cg_one_cta(int n, const int* rowptr, const int* col, const double* val,
@@ -2834,15 +2835,15 @@ __global__ void k_zero_list(T* uI, const int* __restrict__ list, int n) {
   if (q < n) uI[list[q]] = T(0);
 }
 
-// Launches of at most this many CTAs (or work units) may overlap their
+// Launches of at most DEP_MAX_CTAS CTAs (or work units) may overlap their
 // predecessor's end (see launch_next): on levels of up to two waves of CTAs the
 // launch latency counts (one cycle of 2x2x2 sub-cubes refined 5 times 0.66 ->
 // 0.46 ms, 7 times 2.98 -> 2.74 ms, 8 times 15.86 -> 15.60 ms).  Larger ones run
 // without: they gain under 1%, their waiting CTAs keep the other stream's work
 // off the SMs in a recovery, and the flat kernels lose 4% (FP32) to the wait
 // between their index loads and the rest (DEP = false leaves it out).
-constexpr int64_t DEP_MAX_CTAS = 2432;
-// Size that decides it for a launch of `size` CTAs of problem p.
+//
+// dep_size: the size that decides it for a launch of `size` CTAs of problem p.
 inline int64_t dep_size(const ProbArgs& p, int64_t size) { return p.overlap ? size : DEP_MAX_CTAS + 1; }
 
 template <class... P, class... A>
@@ -3755,8 +3756,7 @@ cudaError_t residual(const LevelArgs& L, const ProbArgs& p, const T* u, const T*
   const uint32_t* items = sizeof(T) == 8 ? L.gs_items64 : L.gs_items32;
   if (flat_on(L, p) && items && write_r && !norm) {
     // the residual before a restriction, on levels whose Gauss-Seidel runs
-    // flat: one chunk per CTA (norm launches keep the tile kernel, whose
-    // partial sums per CTA measured faster)
+    // flat: one chunk per CTA
     const int* off = sizeof(T) == 8 ? L.gs_off64 : L.gs_off32;
     const int sk = skip >= 0 && skip < 4 ? skip : -1;
     const int n_items = off[4];
