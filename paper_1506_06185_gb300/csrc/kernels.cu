@@ -848,13 +848,19 @@ __global__ void __launch_bounds__(CTA, 5) k_gs(int N, const int* __restrict__ rs
 // waits for a few CTAs each walking a whole tile; here every thread has one
 // item and the launch lasts about one item's latency.  Same arithmetic per
 // item as gs_tile7, so the iterate equals the tile kernel's bit for bit.
-// Resident CTAs per SM: the FP64 form is held to 8 (32 registers; measured
-// 1.2% faster at refinement 8); the FP32 form is left to the compiler (0: no
-// bound; 3% slower held to 8, 6% slower held to 6).
+// Resident CTAs per SM: the FP64 7-point form is held to 8 (32 registers;
+// measured 1.2% faster at refinement 8); the FP32 form is left to the compiler
+// (0: no bound; 3% slower held to 8, 6% slower held to 6).  Launches that
+// overlap their predecessor keep the interface entries in registers: the FP64
+// 15-point form is held to 3 CTAs (100 registers and 2 CTAs otherwise: solve
+// with moved corners 11.97 instead of 11.71 ms); the FP32 7-point form is not
+// held to 6 (spills: a mixed cycle of 2x2x2 sub-cubes refined 6 times 693
+// instead of 629 us).
 template <class T>
-struct FlatMinCtas {
-  static constexpr int value = sizeof(T) == 8 ? 8 : 0;
-};
+constexpr int flat_min_ctas(bool s7, bool dep) {
+  const bool f64 = sizeof(T) == 8;
+  return !f64 ? 0 : dep ? (s7 ? 0 : 3) : (s7 ? 8 : 0);
+}
 
 // Interface node of a launch that overlaps its predecessor: the stencil entries
 // (all six of the 7-point form, up to 16 else) and the first two copies'
@@ -904,7 +910,7 @@ __device__ __forceinline__ void gs_if_prefetched(const IfTab<T>& tab, int q, int
 }
 
 template <class T, bool S7, bool SCALED, bool DEP>
-__global__ void __launch_bounds__(CTA, S7 && !DEP ? FlatMinCtas<T>::value : 0) k_gs_flat(int N, const int* __restrict__ rs, int64_t block, T* u,
+__global__ void __launch_bounds__(CTA, flat_min_ctas<T>(S7, DEP)) k_gs_flat(int N, const int* __restrict__ rs, int64_t block, T* u,
                                                  T* uI, const T* fI,
                                                  const T* __restrict__ W, const T* __restrict__ Winv,
                                                  const T* fv, const T* __restrict__ Wv,
@@ -1476,15 +1482,17 @@ __global__ void __launch_bounds__(CTA) k_res_flat(int N, const int* __restrict__
     const int j = (int)(d >> 20), k = (int)((d >> 10) & 1023u), g = (int)(d & 1023u);
     const T* w = W + (size_t)macro * 16 * NDIR;
     const size_t mb = (size_t)macro * block;
-    // slice_consts inside each branch: before it the constants stay live through
-    // both, 48 registers instead of 40 and five CTAs per SM instead of six
+    // 7 points: slice_consts inside each branch on the skipped colour: before it
+    // the constants stay live through both, 48 registers instead of 40 and five
+    // CTAs per SM instead of six
     if constexpr (S7) {
       const T wr[11] = {w[0], w[1], w[2], w[3], T(0), T(0), T(0), T(0), w[8], w[9], w[10]};
       if (c == skip) res_group7<T, WRITE, NORM, true>(slice_consts(rs, N, k), N, j, g, c, u + mb, f + mb, r + mb, wr, ss);
       else res_group7<T, WRITE, NORM, false, !DEP>(slice_consts(rs, N, k), N, j, g, c, u + mb, f + mb, r + mb, wr, ss);
     } else {
-      if (c == skip) res_group15<T, WRITE, NORM, true>(slice_consts(rs, N, k), N, j, g, c, u + mb, f + mb, r + mb, w, ss);
-      else res_group15<T, WRITE, NORM, false, !DEP>(slice_consts(rs, N, k), N, j, g, c, u + mb, f + mb, r + mb, w, ss);
+      const Slice sc = slice_consts(rs, N, k);
+      if (c == skip) res_group15<T, WRITE, NORM, true>(sc, N, j, g, c, u + mb, f + mb, r + mb, w, ss);
+      else res_group15<T, WRITE, NORM, false, !DEP>(sc, N, j, g, c, u + mb, f + mb, r + mb, w, ss);
     }
   }
   if (NORM) {
