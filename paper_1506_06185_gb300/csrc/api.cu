@@ -890,10 +890,14 @@ void drop_local_graph(hhg_mesh* m) {
 // Whether Omega_F's launches may overlap each other beside the cycles of the
 // problem `other` on another stream.  Where both sides' finest sweeps fill the
 // GPU the other side is what the recovery waits for, and a denser Omega_F at the
-// higher priority only slows it down (cube refined 8 times, 12 + 3 cycles: the
-// two sides take 29.7 / 60.8 ms with, 35.6 / 55.4 ms without); elsewhere the
-// latency of Omega_F's launches counts (refined 6 times: 5.6 / 5.6 against 6.3 /
-// 2.2 ms; one macro of 3x3x3 sub-cubes in a DN solve: 16.2 against 18.2 ms).
+// higher priority only slows it down (cube refined 8 times, DD: 170.0 ms with,
+// 165.2 without; mixed 103.2 / 99.9); elsewhere the latency of Omega_F's
+// launches counts.  Solves with one recovery (eta = 4, n_I = 3), with / without:
+// 2x2x2 refined 5 times 6.3 / 7.1 ms, 6 times 11.3 / 11.8 (DD) and 10.8 / 12.4
+// (DN); 3x3x3 refined 6 times, one macro lost, 17.3 / 18.5 and 15.8 / 17.4.
+// The line is not the best one everywhere: beside a healthy side of two waves
+// and more DD is slower with (2x2x2 refined 7 times 32.5 / 31.5, 3x3x2 62.6 /
+// 58.5, 4x4x4 refined 6 times 34.4 / 31.6), DN from three waves on.
 int overlap_beside(const hhg_mesh* m, const DevProblem& other) {
   // CTAs of 256 vectors in one colour of one macro: about N^3 / 48 vectors (FP64)
   const int64_t N = m->host.lv.back().N, per_macro = N * N * N / (48 * 256);
