@@ -2264,6 +2264,7 @@ int hhg_walk_counts(hhg_mesh* m, int64_t* counts) {
 
 int hhg_flat_levels(const hhg_mesh* m, int* flat) {
   if (!m || !flat) return fail(HHG_ERR_ARG, "null argument");
+  HHG_TRY(check_device(m));
   for (int l = 0; l < (int)m->host.lv.size(); ++l) flat[l] = flat_on(largs(m, l), pargs(m->global, l)) ? 1 : 0;
   return HHG_OK;
 }
