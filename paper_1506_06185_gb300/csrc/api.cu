@@ -264,6 +264,16 @@ int upload(hhg_mesh* m, T** p, const std::vector<T>& v) {
   return HHG_OK;
 }
 
+// Tables are written on the legacy stream, and the kernels that read them run on
+// the caller's and the mesh's own streams, which may not wait for it: a copy
+// from pageable memory may be under way when the call returns, and so may a
+// clear or a copy within the device.  Every set-up after the mesh's creation
+// ends with this wait.
+int tables_written() {
+  HHG_CUDA(cudaStreamSynchronize(0));
+  return HHG_OK;
+}
+
 void free_all(hhg_mesh* m) {
   for (void* p : m->allocs) cudaFree(p);
   m->allocs.clear();
@@ -466,7 +476,6 @@ int upload_general_if_tables(hhg_mesh* m, DevProblemLevel& q, int l, int kind, c
       HHG_TRY(upload_after(m, &q.tnb, g.tnb, G.entries, nb));
       HHG_TRY(upload_after(m, &q.tw64, g.tw64, G.entries, w));
       if (m->precision == 32) HHG_TRY(upload_after(m, &q.tw32, g.tw32, G.entries, w));
-      HHG_CUDA(cudaStreamSynchronize(0));   // the copies within the device
     }
     ptr.resize(n);
     len.resize(n);
@@ -1070,6 +1079,7 @@ int setup_fault(hhg_mesh* m, const std::vector<unsigned char>& set) {
   HHG_TRY(upload(m, &m->fault_restore_off, off));
   HHG_TRY(upload(m, &m->fault_restore_master, mst));
   m->n_fault_restore = (int)off.size();
+  HHG_TRY(tables_written());
   m->fault_set = set;
   m->has_fault = true;
   return HHG_OK;
@@ -1174,6 +1184,7 @@ int setup_dn(hhg_mesh* m, const std::vector<unsigned char>& set) {
     HHG_CUDA(cudaEventCreateWithFlags(&m->ev_dn_e, cudaEventDisableTiming));
     for (int b = 0; b < 2; ++b) HHG_CUDA(cudaEventCreateWithFlags(&m->ev_dn_r[b], cudaEventDisableTiming));
   }
+  HHG_TRY(tables_written());
   m->dn_set = set;
   m->has_dn = true;
   return HHG_OK;
@@ -1298,7 +1309,7 @@ int update_coefficients(hhg_mesh* m, const double* coeff) {
         HHG_TRY(upload_if_tables(m, d->lv[l], (int)l, d->kind, d->free_host[l], std::vector<int>(),
                                  std::vector<Copy>()));
   }
-  return HHG_OK;
+  return tables_written();
 }
 
 // Candidate shapes of the interior tiles: (nodes of one colour per tile in its
@@ -1365,6 +1376,7 @@ int set_flat(hhg_mesh* m, int l, int mode) {
     HHG_TRY(upload(m, &tb.slot_items, slots));
     tb.n_slots = (int)slots.size();
   }
+  HHG_TRY(tables_written());
   tb.gs_flat = mode;
   return HHG_OK;
 }
@@ -1398,6 +1410,7 @@ int tune_level(hhg_mesh* m, int l, int reps, cudaStream_t s, int* best_out) {
     std::vector<Tile> tiles;
     build_pair_tiles(H.N, tiles, TUNE_CAND[c][0], TUNE_CAND[c][1]);
     HHG_TRY(upload(m, &dev[c], tiles));
+    HHG_TRY(tables_written());
     ndev[c] = (int)tiles.size();
     tb.tiles_int = dev[c];
     tb.n_tiles_int = ndev[c];
@@ -1487,7 +1500,7 @@ int upload_priorities(hhg_batch* b, const std::vector<int>& prio) {
   b->n_seg = (int)seg.size() - 1;
   if (n > 0) HHG_CUDA(cudaMemcpy(b->d_order, order.data(), n * sizeof(int), cudaMemcpyHostToDevice));
   HHG_CUDA(cudaMemcpy(b->d_seg, seg.data(), seg.size() * sizeof(int), cudaMemcpyHostToDevice));
-  return HHG_OK;
+  return tables_written();
 }
 
 // The batch's device is current and its meshes are still there.

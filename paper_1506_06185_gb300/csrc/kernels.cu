@@ -60,7 +60,7 @@ constexpr int CTA = TILE_ROWS * TILE_SLOTS;   // 256 threads, 32 x 8
 // (launch_next lets the successor start as early as that).  after_previous
 // returns when the predecessor has completed and its writes are visible; before
 // it a kernel touches only tables written at set-up (work items, active macros,
-// lists, copy pointers, stencil weights), which host-synchronous copies wrote.
+// lists, copy pointers, stencil weights), whose writing the host waited for.
 // Every kernel calls it, so completion stays in stream order.
 //
 // The vectors (iterates, loads, residuals, partial sums) may change while such
