@@ -61,7 +61,8 @@ constexpr int CTA = TILE_ROWS * TILE_SLOTS;   // 256 threads, 32 x 8
 // returns when the predecessor has completed and its writes are visible; before
 // it a kernel touches only tables written at set-up (work items, active macros,
 // lists, copy pointers, stencil weights), whose writing the host waited for.
-// Every kernel calls it, so completion stays in stream order.
+// Every kernel launched so calls it, and completion stays in stream order; the
+// forms with DEP = false are launched without, after their predecessor's end.
 //
 // The vectors (iterates, loads, residuals, partial sums) may change while such
 // a kernel is resident and waits.  So its vector parameters are not
